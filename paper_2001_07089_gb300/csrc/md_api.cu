@@ -48,8 +48,6 @@ struct md_system {
   double4_32a* d_p4[2] = {nullptr, nullptr};
   double* d_veld = nullptr;
   double* d_frcd = nullptr;
-  double4_32a* d_xbd = nullptr;
-  double4_32a* d_xbd_in = nullptr;
   int32_t* d_gid = nullptr;
   uint8_t* d_typ = nullptr;
   int32_t* d_img = nullptr;
@@ -180,7 +178,7 @@ void dfree(md_system* s, T*& p) {
 __global__ void k_set_state(bool mixed, int ndim, int64_t n_total, int64_t ntot, const RepDev* reps,
                             const int32_t* rep_of, const uint8_t* typ_caller, const double* pos, const double* vel,
                             int cur, uint64_t* pfx, uint4* pq, float* velf, float* frcf, uint4* xbq, double4_32a* p4,
-                            double* veld, double* frcd, double4_32a* xbd, int32_t* gid, uint8_t* typ, int32_t* img) {
+                            double* veld, double* frcd, int32_t* gid, uint8_t* typ, int32_t* img) {
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= n_total) return;
   const RepDev& R = reps[rep_of[g]];
@@ -199,15 +197,15 @@ __global__ void k_set_state(bool mixed, int ndim, int64_t n_total, int64_t ntot,
       frcf[c * ntot + i] = 0.0f;
     }
     pq[i] = make_uint4(hi[0], hi[1], hi[2], t);
-    xbq[i] = pq[i];
   } else {
-    p4[i] = make_double4_32a(x[0], x[1], x[2], (double)t);
-    xbd[i] = p4[i];
+    p4[i] = make_double4_32a(x[0], x[1], x[2], __longlong_as_double((long long)t));
+    pq[i] = kamd::words_of(R.fx32, x[0], x[1], x[2], t);
     for (int c = 0; c < 3; ++c) {
       veld[c * ntot + i] = (vel && (ndim == 3 || c < 2)) ? vel[3 * g + c] : 0.0;
       frcd[c * ntot + i] = 0.0;
     }
   }
+  xbq[i] = pq[i];
   for (int c = 0; c < 3; ++c) img[c * ntot + i] = 0;
   gid[i] = (int32_t)g;
   typ[i] = (uint8_t)t;
@@ -536,6 +534,12 @@ double rc_max(const md_system* s) {
   return m;
 }
 
+// Lanes per particle in the lists: the tuning's, but at least four on the FP64
+// path, whose force phase costs what its FP64 instructions cost: units of eight
+// particles spread them evenly over the SMs (N = 32 000: 26 units per SM
+// instead of 6.6, which left the FP64 pipes 18 % idle).
+int list_lanes(const md_system* s) { return s->mixed ? s->tun.threads_per_atom : std::max(4, s->tun.threads_per_atom); }
+
 // Cells per edge and list capacity follow from the skin; both are recomputed
 // whenever the tuning changes. Cells are at least half the outer list radius
 // wide, so the list build scans the 5 x 5 x 5 cells around a particle's own
@@ -543,6 +547,8 @@ double rc_max(const md_system* s) {
 // a box with fewer than 8 such cells per edge uses cells of the full radius
 // (3 x 3 x 3), and one with fewer than 3 of those an all-pairs scan.
 // KAMD_CELL_REACH=1 keeps cells of the full radius (for tests of that path).
+// Cells are wider than that by more than the 32-bit words, from which particles
+// are binned, lie off the positions.
 void layout_cells(md_system* s) {
   const double rl = rc_max(s) + s->tun.skin_outer;
   int reach = 2;
@@ -551,8 +557,9 @@ void layout_cells(md_system* s) {
   for (int r = 0; r < s->nrep; ++r) {
     RepDev& R = s->reps[r];
     int nr = reach;
-    int nc = (int)std::min(std::floor(R.L / (rl / nr)), 1024.0);
-    const int nc1 = (int)std::floor(R.L / rl);
+    const double off = std::ldexp(R.L, -31);
+    int nc = (int)std::min(std::floor(R.L / (rl / nr + off)), 1024.0);
+    const int nc1 = (int)std::floor(R.L / (rl + off));
     // full-width cells where they fit 3 per edge and half-width cells fewer
     // than 8 (measured on 8 replicas of N = 1000, L = 9.41: 6 half-width
     // cells per edge were 13 % slower than 3 full-width ones), and where the
@@ -567,6 +574,7 @@ void layout_cells(md_system* s) {
     R.nc = nc;
     R.nr = nc > 0 ? nr : 1;
     R.cellw = nc > 0 ? (float)(R.L / nc) : 0.0f;
+    R.mg = s->mixed ? 0.0f : (float)(4.0 * std::sqrt(3.0) * (rl + off) * off);
     R.cell0 = cell0;
     R.cs0 = cell0 + r;
     cell0 += (int64_t)nc * nc * nc;
@@ -616,7 +624,7 @@ void choose_groups(md_system* s) {
       // Groups stop at 64 cells: the staging area of 128-cell groups (57 KB per
       // CTA at N = 10^6) takes shared memory from the L1 cache that the force
       // phase's gathers use (list build 20 % faster, force phase 8 % slower)
-      const double fit = 0.9 * (double)s->tun.block_size / ((double)s->tun.threads_per_atom * occ);
+      const double fit = 0.9 * (double)s->tun.block_size / ((double)list_lanes(s) * occ);
       while (2 * g <= gmax && 2 * g <= fit) g *= 2;
     }
     if (forced) g = forced;
@@ -659,10 +667,15 @@ int stage_capacity(md_system* s) {
   return cap;
 }
 
-size_t stage_bytes(const md_system* s) { return (size_t)s->stage_cap * (s->mixed ? 16 : 36); }
+// Dynamic shared memory of the persistent kernel: the list build's staging area;
+// the FP64 path's force phase uses it for its queues (2 KB per warp).
+size_t stage_bytes(const md_system* s) {
+  const size_t stage = (size_t)s->stage_cap * 16;
+  return s->mixed ? stage : std::max(stage, (size_t)s->tun.block_size / 32 * 2048);
+}
 
 md_status alloc_cells_and_list(md_system* s, int cap_entries) {
-  const int T = s->tun.threads_per_atom;
+  const int T = list_lanes(s);
   dfree(s, s->d_ccount);
   dfree(s, s->d_cstart);
   dfree(s, s->d_ccursor);
@@ -779,17 +792,21 @@ void fill_tables(const md_system* s, KParams& p) {
     const double sr6 = std::pow(sg / rc, 6.0);
     const double vc = 4.0 * e * (sr6 * sr6 - sr6);
     const double rl = rc + s->tun.skin_outer, rli = rc + s->tun.skin;
+    const double s6 = sg * sg * sg * sg * sg * sg;
     p.tab_d[t][0] = rc * rc;
-    p.tab_d[t][1] = sg * sg;
-    p.tab_d[t][2] = 48.0 * e;
-    p.tab_d[t][3] = 4.0 * e;
-    p.vsh_d[t] = vc;
-    p.rl2_d[t] = rl * rl;
-    p.rli2_d[t] = rli * rli;
+    p.tab_d[t][1] = 48.0 * e * s6 * s6;
+    p.tab_d[t][2] = 24.0 * e * s6;
+    p.tab_d[t][3] = vc;
+    p.tabe_d[t][0] = 4.0 * e * s6 * s6;
+    p.tabe_d[t][1] = 4.0 * e * s6;
     p.rli2_f[t] = (float)(rli * rli * (1.0 + 1e-5));
-    for (int k = 0; k < 4; ++k) p.tab_f[t][k] = (float)p.tab_d[t][k];
+    p.rcw2_f[t] = (float)(rc * rc * (1.0 + 1e-5));
+    p.tab_f[t][0] = (float)(rc * rc);
+    p.tab_f[t][1] = (float)(sg * sg);
+    p.tab_f[t][2] = (float)(48.0 * e);
+    p.tab_f[t][3] = (float)(4.0 * e);
     p.vsh_f[t] = (float)vc;
-    // the mixed list test runs in FP32 on cell-relative coordinates: widen the
+    // the list tests run in FP32 on cell-relative coordinates: widen the
     // radius by a relative 1e-5 so rounding can never drop a pair at the edge
     p.rl2_f[t] = (float)(rl * rl * (1.0 + 1e-5));
   }
@@ -803,7 +820,7 @@ KParams make_params(const md_system* s) {
   p.ndim = s->ndim;
   p.ntot = s->ntot;
   p.ntiles = s->ntiles;
-  p.T = s->tun.threads_per_atom;
+  p.T = list_lanes(s);
   p.maxrows = s->maxrows;
   fill_tables(s, p);
   p.mass = s->mass;
@@ -836,8 +853,6 @@ KParams make_params(const md_system* s) {
   p.p4[1] = s->d_p4[1];
   p.veld = s->d_veld;
   p.frcd = s->d_frcd;
-  p.xbd = s->d_xbd;
-  p.xbd_in = s->d_xbd_in;
   p.gid = s->d_gid;
   p.typ = s->d_typ;
   p.img = s->d_img;
@@ -874,7 +889,7 @@ KParams make_params(const md_system* s) {
   p.part[1] = s->d_part[1];
   p.plog = s->d_plog;
   p.plog_rec = s->d_plog_rec;
-  p.plog_stride = (int64_t)s->ntiles * s->tun.threads_per_atom * MD_NPART;
+  p.plog_stride = (int64_t)s->ntiles * p.T * MD_NPART;
   p.plog_slots = (s->plog_slots > 0 && (size_t)s->plog_slots * (size_t)p.plog_stride <= s->plog_cap) ? s->plog_slots : 0;
   return p;
 }
@@ -982,9 +997,9 @@ md_status run_op(md_system* s, int op, int kind, double dt, int64_t nsteps, int6
     }
     if (pend & MD_FLAG_OVERFLOW) {
       // a list column or the build's staging area was too small: grow both
-      const int cap = s->maxrows * s->tun.threads_per_atom;
+      const int cap = s->maxrows * list_lanes(s);
       CKS(alloc_cells_and_list(s, cap + cap / 2 + 16));
-      s->stage_cap = std::min(s->stage_cap + s->stage_cap / 2, (int)(200 * 1024 / (s->mixed ? 16 : 36)));
+      s->stage_cap = std::min(s->stage_cap + s->stage_cap / 2, 200 * 1024 / 16);
       CKS(configure_grid(s));
       CKS(mark_rebuild_all(s));
       continue;
@@ -1052,8 +1067,7 @@ md_status set_state_impl(md_system* s, const double* pos, const double* vel, int
   const int b = 256;
   k_set_state<<<blocks_for(s->n_total, b), b, 0, s->stream>>>(
       s->mixed, s->ndim, s->n_total, s->ntot, s->d_reps, s->d_rep_of_caller, s->d_typ_caller, dpos, dvel, 0, s->d_pfx,
-      s->d_pq[0], s->d_velf, s->d_frcf, s->d_xbq, s->d_p4[0], s->d_veld, s->d_frcd, s->d_xbd, s->d_gid, s->d_typ,
-      s->d_img);
+      s->d_pq[0], s->d_velf, s->d_frcf, s->d_xbq, s->d_p4[0], s->d_veld, s->d_frcd, s->d_gid, s->d_typ, s->d_img);
   CK(cudaGetLastError());
   CK(cudaMemsetAsync(s->d_nnb, 0, sizeof(int32_t) * 8 * (size_t)s->ntot, s->stream));
   CK(cudaMemsetAsync(s->d_nnb_in, 0, sizeof(int32_t) * 8 * (size_t)s->ntot, s->stream));
@@ -1180,6 +1194,7 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
     R.fxs = (float)(L_per[r] / 4294967296.0);
     R.fx64f = (float)R.fx64;
     R.fx32f = (float)(4294967296.0 / L_per[r]);
+    R.fx32 = 4294967296.0 / L_per[r];
     s->reps[r] = R;
     s->out0.push_back(o0);
     for (int t = 0; t < R.ntiles; ++t) tile_rep.push_back(r);
@@ -1201,14 +1216,14 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
   AL(s->d_plog_rec, (size_t)MD_LOG_SLOTS);
   AL(s->d_tile_rep, (size_t)s->ntiles);
   AL(s->d_ctl, 1);
+  AL(s->d_pq[0], nt);
+  AL(s->d_pq[1], nt);
+  AL(s->d_xbq, nt);
+  AL(s->d_xbq_in, nt);
   if (s->mixed) {
     AL(s->d_pfx, 3 * nt);
-    AL(s->d_pq[0], nt);
-    AL(s->d_pq[1], nt);
     AL(s->d_velf, 3 * nt);
     AL(s->d_frcf, 3 * nt);
-    AL(s->d_xbq, nt);
-    AL(s->d_xbq_in, nt);
     AL(s->d_tpfx, 3 * nt);
     float* tv = nullptr;
     float* tf = nullptr;
@@ -1221,8 +1236,6 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
     AL(s->d_p4[1], nt);
     AL(s->d_veld, 3 * nt);
     AL(s->d_frcd, 3 * nt);
-    AL(s->d_xbd, nt);
-    AL(s->d_xbd_in, nt);
     AL(s->d_tp4, nt);
     double* tv = nullptr;
     double* tf = nullptr;
@@ -1359,7 +1372,7 @@ static md_status step_common(md_system* s, int kind, double dt, int64_t nsteps, 
   // Nose-Hoover kinds reduce every step anyway
   int slots = 0;
   if (nlog > 0 && kind != MD_KIND_NH && kind != MD_KIND_NH_EXACT && !s->log_now) {
-    const size_t stride = (size_t)s->ntiles * s->tun.threads_per_atom * MD_NPART;
+    const size_t stride = (size_t)s->ntiles * list_lanes(s) * MD_NPART;
     const size_t most = ((size_t)256 << 20) / sizeof(double) / stride;
     slots = (int)std::min<int64_t>(std::min<int64_t>(nlog, MD_LOG_SLOTS), (int64_t)most);
     if (slots > 0 && (size_t)slots * stride > s->plog_cap) {
@@ -1710,14 +1723,14 @@ md_status md_get_info(md_system* s, md_info* info) {
   CK(cudaMemsetAsync(s->d_count, 0, 8, s->stream));
   // entries of the list the force phase reads: the inner list when there are two
   const bool dual = s->tun.skin_outer > s->tun.skin;
-  k_sum_i32<<<std::max(1, std::min(1024, blocks_for(s->ntot * s->tun.threads_per_atom, 256))), 256, 0, s->stream>>>(
-      s->ntot * s->tun.threads_per_atom, dual ? s->d_nnb_in : s->d_nnb, s->d_count);
+  k_sum_i32<<<std::max(1, std::min(1024, blocks_for(s->ntot * list_lanes(s), 256))), 256, 0, s->stream>>>(
+      s->ntot * list_lanes(s), dual ? s->d_nnb_in : s->d_nnb, s->d_count);
   CK(cudaGetLastError());
   unsigned long long entries = 0;
   CK(cudaMemcpyAsync(&entries, s->d_count, 8, cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   info->list_entries = (int64_t)entries;
-  info->list_capacity = (int64_t)s->maxrows * s->tun.threads_per_atom;
+  info->list_capacity = (int64_t)s->maxrows * list_lanes(s);
   info->device_bytes = (int64_t)s->bytes;
   info->precision = s->mixed ? MD_PREC_MIXED : MD_PREC_FP64;
   info->graph_launches = s->graph_launches;
@@ -1794,8 +1807,8 @@ void md_destroy(md_system* s) {
   drop_graph(s);
   dfree(s, s->d_reps); dfree(s, s->d_tile_rep); dfree(s, s->d_ctl);
   dfree(s, s->d_pfx); dfree(s, s->d_pq[0]); dfree(s, s->d_pq[1]); dfree(s, s->d_velf); dfree(s, s->d_frcf); dfree(s, s->d_xbq);
-  dfree(s, s->d_xbq_in); dfree(s, s->d_xbd_in); dfree(s, s->d_nbr_in); dfree(s, s->d_nnb_in);
-  dfree(s, s->d_p4[0]); dfree(s, s->d_p4[1]); dfree(s, s->d_veld); dfree(s, s->d_frcd); dfree(s, s->d_xbd);
+  dfree(s, s->d_xbq_in); dfree(s, s->d_nbr_in); dfree(s, s->d_nnb_in);
+  dfree(s, s->d_p4[0]); dfree(s, s->d_p4[1]); dfree(s, s->d_veld); dfree(s, s->d_frcd);
   dfree(s, s->d_gid); dfree(s, s->d_typ); dfree(s, s->d_img);
   dfree(s, s->d_tpfx); dfree(s, s->d_tp4); dfree(s, s->d_tvel); dfree(s, s->d_tfrc); dfree(s, s->d_tgid); dfree(s, s->d_ttyp);
   dfree(s, s->d_timg);

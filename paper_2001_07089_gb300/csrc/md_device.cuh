@@ -71,6 +71,16 @@ __device__ __forceinline__ double from_fixed(uint64_t u, double L) {
   return (double)u * (L * (1.0 / 18446744073709551616.0));
 }
 
+// Top 32-bit words of a position in [0, L) (s = 2^32 / L), FP64 path: what the
+// list build, the prune and the cutoff pre-test read. Adding 2^52 leaves the
+// rounded product, mod 2^32, in the low word: one FMA per coordinate. Each word
+// is within L/2^32 of the position; the tests on them are widened by more.
+__device__ __forceinline__ uint4 words_of(double s, double x, double y, double z, uint32_t type) {
+  const double big = 4503599627370496.0;
+  return make_uint4((uint32_t)__double2loint(fma(x, s, big)), (uint32_t)__double2loint(fma(y, s, big)),
+                    (uint32_t)__double2loint(fma(z, s, big)), type);
+}
+
 __device__ __forceinline__ double wrap_box(double x, double L) {
   x -= L * floor(x / L);
   if (x >= L) x -= L;

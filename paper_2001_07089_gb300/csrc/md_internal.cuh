@@ -6,10 +6,12 @@
 //
 //   mixed precision                       all-FP64
 //   pfx   u64  [3][ntot]  fixed point     p4[2] double4_32a [ntot]  (x,y,z,type)
-//   pq[2] uint4 [ntot] (x,y,z hi32,type)  -- gather copy = master, double-buffered
+//   pq[2] uint4 [ntot] (x,y,z hi32,type)  -- gather copy = master, double-buffered; w holds the type's
+//                                         integer bits. pq[2] as in mixed: 32-bit words of the
+//                                         positions, for list tests and the cutoff pre-test
 //   velf  f32  [3][ntot]                  veld f64 [3][ntot]
 //   frcf  f32  [3][ntot]                  frcd f64 [3][ntot]
-//   xbq   uint4 [ntot] (position at the   xbd  double4_32a [ntot]
+//   xbq   uint4 [ntot] (position at the   xbq  as in mixed
 //         last list build, hi32)
 //   gid i32 [ntot] caller index; typ u8 [ntot]; img i32 [3][ntot] image counters
 //   nbr i32 [ntiles][maxrows][32*T]: lane s of particle a of a tile owns
@@ -64,6 +66,8 @@ struct RepDev {
   float fx64f;      // 2^64 / L
   float fx32f;      // 2^32 / L
   float cellw;      // L / nc
+  float mg;         // FP64 path: bound on the error of a squared distance taken from 32-bit words (mixed: 0)
+  double fx32;      // 2^32 / L
   // bath
   double T_target, Q;
   double xi, g, lns, lns_next, xi_a;
@@ -135,10 +139,9 @@ struct KParams {
   float vsh_f[MD_MAXTYPES * MD_MAXTYPES];      // V(rc)
   float rl2_f[MD_MAXTYPES * MD_MAXTYPES];      // outer list radius^2: (rc + skin_outer)^2
   float rli2_f[MD_MAXTYPES * MD_MAXTYPES];     // inner list radius^2: (rc + skin)^2
-  double tab_d[MD_MAXTYPES * MD_MAXTYPES][4];
-  double vsh_d[MD_MAXTYPES * MD_MAXTYPES];
-  double rl2_d[MD_MAXTYPES * MD_MAXTYPES];
-  double rli2_d[MD_MAXTYPES * MD_MAXTYPES];
+  float rcw2_f[MD_MAXTYPES * MD_MAXTYPES];     // rc^2, widened: the FP64 path's pre-test
+  double tab_d[MD_MAXTYPES * MD_MAXTYPES][4];  // rc^2, 48 eps sigma^12, 24 eps sigma^6, V(rc)
+  double tabe_d[MD_MAXTYPES * MD_MAXTYPES][2]; // 4 eps sigma^12, 4 eps sigma^6
   double mass, inv_mass;
   double skin_half2;   // ((skin_outer - skin)/2)^2, one list: (skin/2)^2: move since the build that forces a rebuild
   double prune_half2;  // (skin/2)^2, one list: infinite: move since the last prune that forces a prune
@@ -168,8 +171,6 @@ struct KParams {
   double4_32a* p4[2];
   double* veld;
   double* frcd;
-  double4_32a* xbd;
-  double4_32a* xbd_in;
   int32_t* gid;
   uint8_t* typ;
   int32_t* img;

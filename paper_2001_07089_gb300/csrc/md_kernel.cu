@@ -40,10 +40,9 @@ struct Shared {
   float vshf[MD_MAXTYPES * MD_MAXTYPES];
   float rl2f[MD_MAXTYPES * MD_MAXTYPES];
   float rli2f[MD_MAXTYPES * MD_MAXTYPES];
+  float rcw2f[MD_MAXTYPES * MD_MAXTYPES];
   double4_32a tabd[MD_MAXTYPES * MD_MAXTYPES];
-  double vshd[MD_MAXTYPES * MD_MAXTYPES];
-  double rl2d[MD_MAXTYPES * MD_MAXTYPES];
-  double rli2d[MD_MAXTYPES * MD_MAXTYPES];
+  double2 tabed[MD_MAXTYPES * MD_MAXTYPES];
   double red[16][MD_NPART];
   int scan[32];
   int snap;
@@ -51,6 +50,13 @@ struct Shared {
   // SM-local work layout of this launch (see sm_layout)
   unsigned sm_bits[8];
   int sm_ok, sm_idx, sm_used, sm_cnt, sm_rank;
+};
+
+// FP64 path: each warp's list entries that passed the cutoff pre-test, 32 T
+// places for each of its 32/T particles.
+#define MD_HITS 1024
+struct HitQueue {
+  uint16_t hit[16][MD_HITS];
 };
 
 __device__ __forceinline__ unsigned long long globaltimer() {
@@ -186,6 +192,31 @@ __device__ __forceinline__ void raise_flag(const KParams& p, int f) {
 
 // ------------------------------------------------------------------ drift
 
+// The triggers of a particle whose position now has the top words hi. Outer
+// list: rebuild once a particle moved more than (skin_outer - skin)/2 since
+// the build; inner list: prune once it moved more than skin/2 since the last
+// prune.
+__device__ __forceinline__ void check_moved(const KParams& p, const RepDev& R, int64_t i, const uint32_t hi[3],
+                                            int64_t nstep) {
+  const uint4 xb = p.xbq[i];
+  const float ex = (float)(int)(hi[0] - xb.x) * R.fxs;
+  const float ey = (float)(int)(hi[1] - xb.y) * R.fxs;
+  const float ez = (float)(int)(hi[2] - xb.z) * R.fxs;
+  if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > p.skin_half2f) {
+    p.reps[p.tile_rep[i >> 5]].want_rebuild = 1;
+    raise_flag(p, MD_FLAG_REBUILD);
+  }
+  if (!p.dual) return;
+  const uint4 xp = p.xbq_in[i];
+  const float gx = (float)(int)(hi[0] - xp.x) * R.fxs;
+  const float gy = (float)(int)(hi[1] - xp.y) * R.fxs;
+  const float gz = (float)(int)(hi[2] - xp.z) * R.fxs;
+  if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) > p.prune_half2f) {
+    p.reps[p.tile_rep[i >> 5]].prune_epoch = nstep;
+    raise_flag(p, MD_FLAG_PRUNE);
+  }
+}
+
 // Position update of one particle, mixed path: an FP32 increment is turned
 // into a 64-bit fixed-point step with 32-bit conversions only (x = d 2^32/L,
 // high word floor(x), low word from the fraction) and added to the integer
@@ -219,75 +250,40 @@ __device__ __forceinline__ void drift_mix(const KParams& p, const RepDev& R, int
     hi[c] = (uint32_t)(un >> 32);
   }
   p.pq[cur ^ 1][i] = make_uint4(hi[0], hi[1], hi[2], type);
-  // outer list: rebuild once a particle moved more than (skin_outer - skin)/2
-  // since the build; inner list: prune once it moved more than skin/2 since
-  // the last prune
-  const uint4 xb = p.xbq[i];
-  const float ex = (float)(int)(hi[0] - xb.x) * R.fxs;
-  const float ey = (float)(int)(hi[1] - xb.y) * R.fxs;
-  const float ez = (float)(int)(hi[2] - xb.z) * R.fxs;
-  if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > p.skin_half2f) {
-    p.reps[p.tile_rep[i >> 5]].want_rebuild = 1;
-    raise_flag(p, MD_FLAG_REBUILD);
-  }
-  if (!p.dual) return;
-  const uint4 xp = p.xbq_in[i];
-  const float gx = (float)(int)(hi[0] - xp.x) * R.fxs;
-  const float gy = (float)(int)(hi[1] - xp.y) * R.fxs;
-  const float gz = (float)(int)(hi[2] - xp.z) * R.fxs;
-  if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) > p.prune_half2f) {
-    p.reps[p.tile_rep[i >> 5]].prune_epoch = nstep;
-    raise_flag(p, MD_FLAG_PRUNE);
-  }
+  check_moved(p, R, i, hi, nstep);
 }
 
-// Position update of one particle, FP64 path: wrap into [0, L).
+// Position update of one particle, FP64 path: wrap into [0, L). Comparisons
+// are made on the bit patterns (of non-negative doubles they order alike): an
+// FP64 compare would cost as much as an FMA of that pipe.
 __device__ __forceinline__ void drift_f64(const KParams& p, const RepDev& R, int64_t i, int cur, const double v[3],
                                           const double a[3], double xi, int64_t nstep) {
   const int64_t nt = p.ntot;
   const double dt = p.dt, hdt2 = 0.5 * p.dt * p.dt;
   const double4_32a x = p.p4[cur][i];
+  const long long lim = __double_as_longlong(0.25 * R.L), Lb = __double_as_longlong(R.L);
   double d[3];
   bool bad = false;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     d[c] = v[c] * dt + (a[c] - xi * v[c]) * hdt2;
-    bad |= !(fabs(d[c]) < 0.25 * R.L);
+    bad |= !((__double_as_longlong(d[c]) & 0x7fffffffffffffffll) < lim);  // (a NaN's pattern is above infinity's)
   }
   if (bad) { raise_flag(p, MD_FLAG_UNSTABLE); return; }
   double xs[3] = {x.x + d[0], x.y + d[1], x.z + d[2]};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    if (xs[c] >= R.L) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
-    else if (xs[c] < 0.0) {
+    if (__double_as_longlong(xs[c]) >= Lb) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
+    else if (__double_as_longlong(xs[c]) < 0) {
       xs[c] += R.L; p.img[c * nt + i] -= 1;
-      if (xs[c] >= R.L) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
+      if (__double_as_longlong(xs[c]) >= Lb) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
     }
   }
   p.p4[cur ^ 1][i] = make_double4_32a(xs[0], xs[1], xs[2], x.w);
-  const double4_32a xb = p.xbd[i];
-  double e[3] = {xs[0] - xb.x, xs[1] - xb.y, xs[2] - xb.z};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (e[c] > 0.5 * R.L) e[c] -= R.L;
-    else if (e[c] < -0.5 * R.L) e[c] += R.L;
-  }
-  if (e[0] * e[0] + e[1] * e[1] + e[2] * e[2] > p.skin_half2) {
-    p.reps[p.tile_rep[i >> 5]].want_rebuild = 1;
-    raise_flag(p, MD_FLAG_REBUILD);
-  }
-  if (!p.dual) return;
-  const double4_32a xp = p.xbd_in[i];
-  double g[3] = {xs[0] - xp.x, xs[1] - xp.y, xs[2] - xp.z};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (g[c] > 0.5 * R.L) g[c] -= R.L;
-    else if (g[c] < -0.5 * R.L) g[c] += R.L;
-  }
-  if (g[0] * g[0] + g[1] * g[1] + g[2] * g[2] > p.prune_half2) {
-    p.reps[p.tile_rep[i >> 5]].prune_epoch = nstep;
-    raise_flag(p, MD_FLAG_PRUNE);
-  }
+  const uint4 u = words_of(R.fx32, xs[0], xs[1], xs[2], (uint32_t)__double2loint(x.w));
+  p.pq[cur ^ 1][i] = u;
+  const uint32_t hi[3] = {u.x, u.y, u.z};
+  check_moved(p, R, i, hi, nstep);
 }
 
 // Stand-alone position update for every particle (first step of a call,
@@ -394,6 +390,113 @@ __device__ __forceinline__ void lane_sum_mix(const Shared& sh, const uint4* __re
   if (r > 2) pair_mix<ENERGY>(sh, pi, pq[jq.z], tb, sc, fx, fy, fz, pe, vir);
 }
 
+// 1/x in FP64: the hardware's 20-bit estimate y and one step of the cubically
+// convergent iteration y (1 + e + e^2), e = 1 - x y: e^3 < 2^-60.
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// Minimum image of one coordinate difference (the branch rule; the comparison
+// is made on the bit patterns of non-negative doubles).
+__device__ __forceinline__ double image_f64(double d, double L, long long hLb) {
+  if ((__double_as_longlong(d) & 0x7fffffffffffffffll) > hLb) d -= copysign(L, d);
+  return d;
+}
+
+// Pair term for one list entry (FP64 path), Eq. (KAFix) and Eq. (VshiftedKALJ)
+// with sigma folded into the constants (16 FP64 operations without energy, 12
+// of them FMAs or multiplies of the pair itself).
+template <bool ENERGY>
+__device__ __forceinline__ void pair_f64(const Shared& sh, const double4_32a& pi, const double4_32a& pj, int tt, double L,
+                                         long long hLb, double& fx, double& fy, double& fz, double& pe, double& vir) {
+  const double dx = image_f64(pi.x - pj.x, L, hLb), dy = image_f64(pi.y - pj.y, L, hLb), dz = image_f64(pi.z - pj.z, L, hLb);
+  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+  const double4_32a c = sh.tabd[tt];
+  if (__double_as_longlong(r2) < __double_as_longlong(c.x)) {
+    const double y = rcp_f64(r2);
+    const double y3 = y * y * y;
+    const double w = y3 * fma(c.y, y3, -c.z);
+    const double fr = w * y;
+    fx = fma(fr, dx, fx);
+    fy = fma(fr, dy, fy);
+    fz = fma(fr, dz, fz);
+    if (ENERGY) {
+      const double2 ce = sh.tabed[tt];
+      pe += fma(y3, fma(ce.x, y3, -ce.y), -c.w);
+      vir += w;
+    }
+  }
+}
+
+// Pair sums of one unit (FP64 path). GB300 issues a warp's FP64 instruction in
+// 16 to 19 cycles of an SM (64 to 76 of its quarter, however many warps there
+// are), so the phase costs what its FP64 instructions cost and nothing else
+// matters. Every list entry is therefore tested in FP32 first, on the 32-bit
+// words and against the cutoff widened by more than the words' and FP32's
+// error (about two thirds pass); the T lanes of a particle queue the entries
+// that pass (by ballots, in list order) and then deal them out evenly, so that
+// the lanes are busy in the FP64 part, which applies the exact cutoff.
+// lp: this lane's column of cnt entries; every lane of the warp takes part.
+template <bool ENERGY>
+__device__ __forceinline__ void unit_sum_f64(const KParams& p, const Shared& sh, const RepDev& R, int cur, const int* lp,
+                                             int64_t i, int cnt, int T, int s, double& fx, double& fy, double& fz,
+                                             double& pe, double& vir) {
+  extern __shared__ __align__(32) unsigned char dyn[];
+  const int lane = threadIdx.x & 31;
+  const int tsh = __ffs(T) - 1, gsz = 32 * T, cap = 32 * T;
+  uint16_t* const queue = reinterpret_cast<HitQueue*>(dyn)->hit[threadIdx.x >> 5] + (lane >> tsh) * cap;
+  const unsigned group = ((1u << T) - 1u) << (lane & ~(T - 1));
+  const unsigned before = group & ((1u << lane) - 1u);
+  const uint4* __restrict__ pq = p.pq[cur];
+  const double4_32a* __restrict__ p4 = p.p4[cur];
+  const uint4 qi = pq[i];
+  const double4_32a pi = p4[i];
+  const int tb = (int)qi.w * p.ntypes;
+  const float sc = R.fxs, mg = R.mg;
+  const double L = R.L;
+  const long long hLb = __double_as_longlong(0.5 * R.L);
+  const int rows = __reduce_max_sync(0xffffffffu, (cnt + 3) >> 2);
+  int held = 0, row0 = 0;  // queued entries of this particle; the row that their places count from
+  int4 jq = make_int4(0, 0, 0, 0);
+  if (cnt > 0) jq = __ldcs(reinterpret_cast<const int4*>(lp));
+  for (int r = 0; r < rows; ++r) {
+    const int j[4] = {jq.x, jq.y, jq.z, jq.w};
+    uint4 pj[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (4 * r + u < cnt) pj[u] = pq[j[u]];
+    if (4 * r + 4 < cnt) jq = __ldcs(reinterpret_cast<const int4*>(lp + (int64_t)(r + 1) * 4 * gsz));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      bool hit = false;
+      if (4 * r + u < cnt) {
+        const float dx = (float)(int)(qi.x - pj[u].x) * sc, dy = (float)(int)(qi.y - pj[u].y) * sc,
+                    dz = (float)(int)(qi.z - pj[u].z) * sc;
+        hit = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) - mg < sh.rcw2f[tb + (int)pj[u].w];
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (hit) queue[held + __popc(m & before)] = (uint16_t)((4 * (r - row0) + u) * T + s);
+      held += __popc(m & group);
+    }
+    // work the queues off at the end, or before a further row could overflow one
+    if (r + 1 < rows && !__any_sync(0xffffffffu, held > cap - 4 * T) && 4 * (r + 2 - row0) * T <= 65536) continue;
+    __syncwarp();
+    for (int k = s; k < held; k += T) {
+      const int e = queue[k];
+      const int q = 4 * row0 + (e >> tsh);  // place in the column of lane e % T
+      const int jj = lp[list_at(4 * ((e & (T - 1)) - s), q, gsz)];
+      const double4_32a pj4 = p4[jj];
+      pair_f64<ENERGY>(sh, pi, pj4, tb + __double2loint(pj4.w), L, hLb, fx, fy, fz, pe, vir);
+    }
+    __syncwarp();
+    held = 0;
+    row0 = r + 1;
+  }
+}
+
 // Force phase. The work unit is one warp: 32/T particles of one tile with T
 // lanes each (a tile of 32 particles is T units). Lane s of particle a walks
 // its own column of the list; the T lanes are combined by a fixed xor tree;
@@ -494,41 +597,20 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
     } else {
       const RepDev* R = &p.reps[p.tile_rep[tile]];
       const bool act = (tile - R->tile0) * 32 + a < R->n;
-      const int cnt = (act && pairs) ? p.nnb_in[i * T + s] : 0;
       double fx = 0, fy = 0, fz = 0, pe = 0, vir = 0;
-      if (act) {
-        const double4_32a* __restrict__ p4 = p.p4[cur];
-        const double4_32a pi = p4[i];
-        const int tb = (int)pi.w * p.ntypes;
-        const double L = R->L, hL = 0.5 * R->L;
-        for (int q = 0; q < cnt; ++q) {
-          const int j = __ldcs(lp + list_at(0, q, gsz));
-          const double4_32a pj = p4[j];
-          double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-          if (dx > hL) dx -= L; else if (dx < -hL) dx += L;
-          if (dy > hL) dy -= L; else if (dy < -hL) dy += L;
-          if (dz > hL) dz -= L; else if (dz < -hL) dz += L;
-          const double r2 = dx * dx + dy * dy + dz * dz;
-          const int tt = tb + (int)pj.w;
-          const double4_32a c = sh.tabd[tt];
-          if (r2 < c.x) {
-            const double ir2 = 1.0 / r2;
-            const double s2 = c.y * ir2;
-            const double s6 = s2 * s2 * s2;
-            const double w = c.z * s6 * (s6 - 0.5);
-            const double fr = w * ir2;
-            fx += fr * dx; fy += fr * dy; fz += fr * dz;
-            pe += c.w * s6 * (s6 - 1.0) - sh.vshd[tt];
-            vir += w;
-          }
-        }
+      if (pairs) {
+        const int cnt = act ? p.nnb_in[i * T + s] : 0;
+        if (energy) unit_sum_f64<true>(p, sh, *R, cur, lp, i, cnt, T, s, fx, fy, fz, pe, vir);
+        else unit_sum_f64<false>(p, sh, *R, cur, lp, i, cnt, T, s, fx, fy, fz, pe, vir);
       }
       for (int o = T >> 1; o > 0; o >>= 1) {
         fx += __shfl_xor_sync(0xffffffffu, fx, o);
         fy += __shfl_xor_sync(0xffffffffu, fy, o);
         fz += __shfl_xor_sync(0xffffffffu, fz, o);
-        pe += __shfl_xor_sync(0xffffffffu, pe, o);
-        vir += __shfl_xor_sync(0xffffffffu, vir, o);
+        if (energy) {
+          pe += __shfl_xor_sync(0xffffffffu, pe, o);
+          vir += __shfl_xor_sync(0xffffffffu, vir, o);
+        }
       }
       double e[6] = {0, 0, 0, 0, 0, 0};
       if (act && s == 0) {
@@ -627,11 +709,12 @@ __device__ void prune_phase(const KParams& p, Shared& sh, int cur, int64_t epoch
     const int cnt = p.nnb[i * T + s];
     int k = 0;
     int b1 = 0, b2 = 0, b3 = 0;  // quad shift register of the list writer
-    if constexpr (MIX) {
+    {
+      // both paths compare 32-bit words (FP64: with the words' margin)
       const uint4* __restrict__ pq = p.pq[cur];
       const uint4 pi = pq[i];
       const int tb = (int)pi.w * p.ntypes;
-      const float sc = R.fxs;
+      const float sc = R.fxs, mg = MIX ? 0.0f : R.mg;
       // a quad of outer entries per iteration: one 16-byte index load, issued
       // a quad ahead, and four position gathers in flight together
       const int64_t qstride = 4 * (int64_t)gsz;
@@ -649,27 +732,11 @@ __device__ void prune_phase(const KParams& p, Shared& sh, int cur, int64_t epoch
           const float dx = (float)(int)(pi.x - pj[u].x) * sc;
           const float dy = (float)(int)(pi.y - pj[u].y) * sc;
           const float dz = (float)(int)(pi.z - pj[u].z) * sc;
-          if (u < m && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < sh.rli2f[tb + (int)pj[u].w])
+          if (u < m && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) - mg < sh.rli2f[tb + (int)pj[u].w])
             list_push(li, gsz, p.maxrows, k, b1, b2, b3, j[u]);
         }
       }
       if (s == 0) p.xbq_in[i] = pi;
-    } else {
-      const double4_32a* __restrict__ p4 = p.p4[cur];
-      const double4_32a pi = p4[i];
-      const int tb = (int)pi.w * p.ntypes;
-      const double L = R.L, hL = 0.5 * R.L;
-      for (int q = 0; q < cnt; ++q) {
-        const int j = __ldcs(lo + list_at(0, q, gsz));
-        const double4_32a pj = p4[j];
-        double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-        if (dx > hL) dx -= L; else if (dx < -hL) dx += L;
-        if (dy > hL) dy -= L; else if (dy < -hL) dy += L;
-        if (dz > hL) dz -= L; else if (dz < -hL) dz += L;
-        if (dx * dx + dy * dy + dz * dz < sh.rli2d[tb + (int)pj.w])
-          list_push(li, gsz, p.maxrows, k, b1, b2, b3, j);
-      }
-      if (s == 0) p.xbd_in[i] = pi;
     }
     list_flush(li, gsz, p.maxrows, k, b1, b2, b3);
     p.nnb_in[i * T + s] = k;
@@ -905,22 +972,14 @@ __device__ __noinline__ void reduce_scalars(const KParams& p, RepDev& R, int64_t
 
 // ------------------------------------------------------------------ rebuild
 
-template <bool MIX>
+// Cell of a particle, from its 32-bit words (both paths).
 __device__ __forceinline__ void cell_of_pos(const KParams& p, const RepDev& R, int64_t i, int cur, int& cx, int& cy,
                                             int& cz) {
   const int nc = R.nc;
-  if constexpr (MIX) {
-    const uint4 q = p.pq[cur][i];
-    cx = (int)(((uint64_t)q.x * (uint64_t)nc) >> 32);
-    cy = (int)(((uint64_t)q.y * (uint64_t)nc) >> 32);
-    cz = (int)(((uint64_t)q.z * (uint64_t)nc) >> 32);
-  } else {
-    const double4_32a x = p.p4[cur][i];
-    const double s = (double)nc * R.invL;
-    cx = min(max((int)(x.x * s), 0), nc - 1);
-    cy = min(max((int)(x.y * s), 0), nc - 1);
-    cz = min(max((int)(x.z * s), 0), nc - 1);
-  }
+  const uint4 q = p.pq[cur][i];
+  cx = (int)(((uint64_t)q.x * (uint64_t)nc) >> 32);
+  cy = (int)(((uint64_t)q.y * (uint64_t)nc) >> 32);
+  cz = (int)(((uint64_t)q.z * (uint64_t)nc) >> 32);
 }
 
 // Block-wide exclusive scan of one int per thread.
@@ -970,29 +1029,26 @@ __device__ __forceinline__ float lim_of(float l0, float l1, float l2, float l3, 
 // REL: staged FP32 coordinates relative to the group's reference particle;
 // otherwise staged fixed-point words and exact integer differences.
 template <bool REL, bool NT2>
-__device__ __forceinline__ unsigned chunk_mask(uint32_t st_s, int q0, int nq, int tsh, float x, float y, float z,
+__device__ __forceinline__ unsigned chunk_mask(const uint4* st, int q0, int nq, int tsh, float x, float y, float z,
                                                const uint4& pq, float sc, float l0, float l1, float l2, float l3) {
   unsigned mask = 0u;
 #pragma unroll 4
   for (int u = 0; u < nq; ++u) {
-    uint32_t c0, c1, c2, c3;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(c0), "=r"(c1), "=r"(c2), "=r"(c3)
-                 : "r"(st_s + 16u * (uint32_t)(q0 + (u << tsh))));
+    const uint4 c = st[q0 + (u << tsh)];
     float dx, dy, dz;
     if constexpr (REL) {
-      dx = x - __uint_as_float(c0);
-      dy = y - __uint_as_float(c1);
-      dz = z - __uint_as_float(c2);
+      dx = x - __uint_as_float(c.x);
+      dy = y - __uint_as_float(c.y);
+      dz = z - __uint_as_float(c.z);
     } else {
-      dx = (float)(int)(pq.x - c0) * sc;
-      dy = (float)(int)(pq.y - c1) * sc;
-      dz = (float)(int)(pq.z - c2) * sc;
+      dx = (float)(int)(pq.x - c.x) * sc;
+      dy = (float)(int)(pq.y - c.y) * sc;
+      dz = (float)(int)(pq.z - c.z) * sc;
     }
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
     // hit: r2 - lim < 0 (the sign of a rounded difference is that of the
     // exact one, and equal values give +0), shifted in from the top
-    const float d = r2 - lim_of<NT2>(l0, l1, l2, l3, c3);
+    const float d = r2 - lim_of<NT2>(l0, l1, l2, l3, c.w);
     mask = (mask >> 1) | (__float_as_uint(d) & 0x80000000u);
   }
   return nq > 0 ? mask >> (32 - nq) : 0u;  // candidate u at bit u
@@ -1004,21 +1060,20 @@ __device__ __forceinline__ unsigned chunk_mask(uint32_t st_s, int q0, int nq, in
 // particle itself is then cleared by index, and a second pass stores the
 // marked candidates in order, reading only their slot words.
 template <bool REL, bool NT2>
-__device__ __forceinline__ int scan_run_mix(uint32_t st_s, int qs, int qe, int tsh, float x, float y, float z,
+__device__ __forceinline__ int scan_run_mix(const uint4* st, int qs, int qe, int tsh, float x, float y, float z,
                                             const uint4& pq, float sc, float l0, float l1, float l2, float l3,
                                             int own_q, int32_t* col, int gsz, int maxrows, int k, int& b1, int& b2,
                                             int& b3) {
   const int T = 1 << tsh;
   for (int q0 = qs; q0 < qe; q0 += 32 << tsh) {
     const int nq = min(32, (qe - q0 + T - 1) >> tsh);
-    unsigned mask = chunk_mask<REL, NT2>(st_s, q0, nq, tsh, x, y, z, pq, sc, l0, l1, l2, l3);
+    unsigned mask = chunk_mask<REL, NT2>(st, q0, nq, tsh, x, y, z, pq, sc, l0, l1, l2, l3);
     const int d = own_q - q0;
     if (d >= 0 && (d & (T - 1)) == 0 && (d >> tsh) < nq) mask &= ~(1u << (d >> tsh));
     while (mask) {
       const int u = __ffs(mask) - 1;
       mask &= mask - 1u;
-      uint32_t w;
-      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(st_s + 16u * (uint32_t)(q0 + (u << tsh)) + 12u));
+      const uint32_t w = st[q0 + (u << tsh)].w;
       list_push(col, gsz, maxrows, k, b1, b2, b3, (int)(w & 0x3fffffffu));
     }
   }
@@ -1038,14 +1093,14 @@ __device__ __forceinline__ float face_dist(int o, float f, float w) {
 // cell of the particle's own cell; (fx, fy, fz): its position inside that
 // cell. Returns the entries found; b1..b3 hold the writer's partial quad.
 template <bool REL, bool NT2>
-__device__ __forceinline__ int scan_particle_mix(uint32_t st_s, const int* s_ub, int ncand, int nc, int nr, int UX,
+__device__ __forceinline__ int scan_particle_mix(const uint4* st, const int* s_ub, int ncand, int nc, int nr, int UX,
                                                  int UY, int u_own, float fx, float fy, float fz, float wc,
                                                  float lcut, int sl, int tsh, float x, float y, float z,
                                                  const uint4& pq, float sc, float l0, float l1, float l2, float l3,
                                                  int own_q, int32_t* col, int gsz, int maxrows, int& b1, int& b2,
                                                  int& b3) {
   if (nc == 0)
-    return scan_run_mix<REL, NT2>(st_s, sl, ncand, tsh, x, y, z, pq, sc, l0, l1, l2, l3, own_q, col, gsz, maxrows, 0,
+    return scan_run_mix<REL, NT2>(st, sl, ncand, tsh, x, y, z, pq, sc, l0, l1, l2, l3, own_q, col, gsz, maxrows, 0,
                                   b1, b2, b3);
   // distances along x to the cells at the ends of a row (nr <= 2)
   const float em2 = fx + wc, em1 = fx, ep1 = wc - fx, ep2 = (wc - fx) + wc;
@@ -1062,7 +1117,7 @@ __device__ __forceinline__ int scan_particle_mix(uint32_t st_s, const int* s_ub,
       if (xh == 2 && fmaf(ep2, ep2, d2) >= lcut) xh = 1;
       if (xh == 1 && fmaf(ep1, ep1, d2) >= lcut) xh = 0;
       const int us0 = u_own + (oz * UY + oy) * UX;  // the row's cell in the particle's own column
-      k = scan_run_mix<REL, NT2>(st_s, s_ub[us0 + xl] + sl, s_ub[us0 + xh + 1], tsh, x, y, z, pq, sc, l0, l1, l2,
+      k = scan_run_mix<REL, NT2>(st, s_ub[us0 + xl] + sl, s_ub[us0 + xh + 1], tsh, x, y, z, pq, sc, l0, l1, l2,
                                  l3, own_q, col, gsz, maxrows, k, b1, b2, b3);
     }
   }
@@ -1078,7 +1133,7 @@ __device__ __forceinline__ int scan_particle_mix(uint32_t st_s, const int* s_ub,
 // gaps, in an order fixed by the data. Returns the column's length (the same
 // on both lanes).
 template <bool REL, bool NT2>
-__device__ __forceinline__ int scan_particle_pair_mix(uint32_t st_s, const int* s_ub, int nr, int UX, int UY,
+__device__ __forceinline__ int scan_particle_pair_mix(const uint4* st, const int* s_ub, int nr, int UX, int UY,
                                                       int u_own, float fx, float fy, float fz, float wc, float lcut,
                                                       int h, unsigned pmask, float x, float y, float z,
                                                       const uint4& pq, float sc, float l0, float l1, float l2,
@@ -1116,7 +1171,7 @@ __device__ __forceinline__ int scan_particle_pair_mix(uint32_t st_s, const int* 
     const int base = q0;
     if (have) {
       const int nq = min(32, qe - q0);
-      mask = chunk_mask<REL, NT2>(st_s, q0, nq, 0, x, y, z, pq, sc, l0, l1, l2, l3);
+      mask = chunk_mask<REL, NT2>(st, q0, nq, 0, x, y, z, pq, sc, l0, l1, l2, l3);
       const int d = own_q - q0;
       if (d >= 0 && d < nq) mask &= ~(1u << d);
       q0 += nq;
@@ -1128,8 +1183,7 @@ __device__ __forceinline__ int scan_particle_pair_mix(uint32_t st_s, const int* 
     while (mask) {
       const int u = __ffs(mask) - 1;
       mask &= mask - 1u;
-      uint32_t w;
-      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(st_s + 16u * (uint32_t)(base + u) + 12u));
+      const uint32_t w = st[base + u].w;
       if (e < maxrows) col[list_at(0, e, gsz)] = (int)(w & 0x3fffffffu);
       ++e;
     }
@@ -1151,14 +1205,10 @@ __device__ __forceinline__ int scan_particle_pair_mix(uint32_t st_s, const int* 
 // than in 27 cells of full width). List column s takes the run entries s,
 // s + T, s + 2T, ... of every row. A replica too small for cells is one group
 // whose single staged "cell" is the whole replica.
-template <bool MIX>
 __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cur) {
   const int T = p.T, gsz = 32 * T;
   extern __shared__ __align__(32) unsigned char dyn[];
   const int stage_cap = p.stage_cap;
-  double4_32a* st_d = reinterpret_cast<double4_32a*>(dyn);  // FP64: positions, then slots
-  int32_t* st_j = reinterpret_cast<int32_t*>(dyn + (size_t)stage_cap * 32);
-  float4* st_f = reinterpret_cast<float4*>(dyn);
   uint4* st_u = reinterpret_cast<uint4*>(dyn);
   // union cells: first slot, staged base; group rows (ly, lz): first slot,
   // particle count prefix
@@ -1266,78 +1316,59 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
       __syncthreads();
       continue;
     }
-    // mixed path with enough cells per edge: stage coordinates relative to a
-    // particle of the group as FP32 (exact integer differences, converted once
+    // with enough cells per edge: stage coordinates relative to a particle of
+    // the group as FP32 (exact integer differences, converted once
     // per candidate). Every staged candidate then lies within (G + nr) cells
     // of the reference along each axis, less than half the box, so
     // differences of relative coordinates are the minimum image; the list
     // test has a whole skin of margin, so FP32 is ample. Otherwise the
     // fixed-point words are staged and every test takes the exact integer
     // difference.
-    const bool rel = MIX && nc >= 2 * (GX + nr) + 1 && nc >= 2 * (GY + nr) + 1 && nc >= 2 * (GZ + nr) + 1;
-    uint4 ref = make_uint4(0u, 0u, 0u, 0u);
-    if constexpr (MIX) ref = p.pq[cur][s_ref];
+    const bool rel = nc >= 2 * (GX + nr) + 1 && nc >= 2 * (GY + nr) + 1 && nc >= 2 * (GZ + nr) + 1;
+    const uint4 ref = p.pq[cur][s_ref];
     {
-      constexpr int STAGE_U = 2;
+      // two candidates per thread and turn, both loads in flight together. (The
+      // loads are made whether or not there is a second candidate: with them
+      // under a condition, in an array, the compiler left the type word of the
+      // second one unset in some instances of this code, and candidates of type
+      // 1 were held to the radius of type 0.)
       const uint4* __restrict__ pqc = p.pq[cur];
-      const double4_32a* __restrict__ p4c = p.p4[cur];
-      for (int t0 = threadIdx.x; t0 < ncand; t0 += STAGE_U * blockDim.x) {
-        int src[STAGE_U];
-#pragma unroll
-        for (int u = 0; u < STAGE_U; ++u) {
-          const int t = t0 + u * (int)blockDim.x;
-          src[u] = -1;
-          if (t < ncand) {
-            int lo = 0, hi = nu;  // s_ub[lo] <= t < s_ub[hi]
-            while (hi - lo > 1) {
-              const int mid = (lo + hi) >> 1;
-              if (s_ub[mid] <= t) lo = mid; else hi = mid;
-            }
-            src[u] = s_ulo[lo] + (t - s_ub[lo]);
-          }
+      const float sc = R.fxs;
+      const int B = (int)blockDim.x;
+      auto slot_of = [&](int t) {
+        int lo = 0, hi = nu;  // s_ub[lo] <= t < s_ub[hi]
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (s_ub[mid] <= t) lo = mid; else hi = mid;
         }
-        if constexpr (MIX) {
-          uint4 q[STAGE_U];
-#pragma unroll
-          for (int u = 0; u < STAGE_U; ++u)
-            if (src[u] >= 0) q[u] = pqc[src[u]];
-          const float sc = R.fxs;
-#pragma unroll
-          for (int u = 0; u < STAGE_U; ++u) {
-            if (src[u] < 0) continue;
-            const int t = t0 + u * (int)blockDim.x;
-            const unsigned w = (q[u].w << 30) | (unsigned)src[u];
-            if (rel)
-              st_f[t] = make_float4((float)(int)(q[u].x - ref.x) * sc, (float)(int)(q[u].y - ref.y) * sc,
-                                    (float)(int)(q[u].z - ref.z) * sc, __int_as_float((int)w));
-            else
-              st_u[t] = make_uint4(q[u].x, q[u].y, q[u].z, w);
-          }
-        } else {
-          double4_32a q[STAGE_U];
-#pragma unroll
-          for (int u = 0; u < STAGE_U; ++u)
-            if (src[u] >= 0) q[u] = p4c[src[u]];
-#pragma unroll
-          for (int u = 0; u < STAGE_U; ++u) {
-            if (src[u] < 0) continue;
-            const int t = t0 + u * (int)blockDim.x;
-            st_d[t] = q[u];
-            st_j[t] = src[u];
-          }
-        }
+        return s_ulo[lo] + (t - s_ub[lo]);
+      };
+      auto stage = [&](int t, const uint4& q, int src) {
+        const unsigned w = (q.w << 30) | (unsigned)src;
+        if (rel)
+          st_u[t] = make_uint4(__float_as_uint((float)(int)(q.x - ref.x) * sc),
+                               __float_as_uint((float)(int)(q.y - ref.y) * sc),
+                               __float_as_uint((float)(int)(q.z - ref.z) * sc), w);
+        else
+          st_u[t] = make_uint4(q.x, q.y, q.z, w);
+      };
+      for (int t0 = threadIdx.x; t0 < ncand; t0 += 2 * B) {
+        const int t1 = t0 + B;
+        const int sa = slot_of(t0), sb = slot_of(min(t1, ncand - 1));
+        const uint4 qa = pqc[sa], qb = pqc[sb];
+        stage(t0, qa, sa);
+        if (t1 < ncand) stage(t1, qb, sb);
       }
     }
     __syncthreads();
     // scan: T threads per particle, particles of the group in row order; with
-    // T = 1 and at most half as many particles as threads (mixed path, cells),
-    // two lanes per particle (scan_particle_pair_mix)
-    const bool pair = MIX && T == 1 && nc > 0 && 2 * npart <= (int)blockDim.x;
+    // T = 1 and at most half as many particles as threads (with cells), two
+    // lanes per particle (scan_particle_pair_mix)
+    const bool pair = T == 1 && nc > 0 && 2 * npart <= (int)blockDim.x;
     const int lanes = pair ? 2 : T;
     const int per_pass = (int)blockDim.x / lanes;
     const int sl = pair ? 0 : (int)threadIdx.x % T;
     const int h = pair ? (int)(threadIdx.x & 1u) : 0;
-    const int side = 2 * nr + 1;  // stencil cells per axis
     for (int pidx = (int)threadIdx.x / lanes; pidx < npart && (int)threadIdx.x < per_pass * lanes;
          pidx += per_pass) {
       int row = 0;
@@ -1346,7 +1377,7 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
       const int ly = row % GY, lz = row / GY;
       // the particle's own cell (the binning of B1) and its position inside it
       int ccx = 0, ccy = 0, ccz = 0;
-      if (nc > 0) cell_of_pos<MIX>(p, R, i, cur, ccx, ccy, ccz);
+      if (nc > 0) cell_of_pos(p, R, i, cur, ccx, ccy, ccz);
       const int lx = ccx - cx;
       // own staged position (each particle is a candidate of its own cell)
       const int own_u = nc > 0 ? ((lz + nr) * UY + (ly + nr)) * UX + (lx + nr) : 0;
@@ -1354,8 +1385,7 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
       int32_t* lb = p.nbr + list_col(i >> 5, p.maxrows, T, (int)(i & 31) * T + sl);
       int k = 0;
       int b1 = 0, b2 = 0, b3 = 0;  // quad shift register of the list writer
-      const int nruns = nc > 0 ? side * side : 1;
-      if constexpr (MIX) {
+      {
         const uint4 pq_i = p.pq[cur][i];
         const float sc = R.fxs;
         const float x = (float)(int)(pq_i.x - ref.x) * sc;
@@ -1364,9 +1394,11 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
         // this particle's row of pair list radii^2, by partner type
         const float* rl = sh.rl2f + (int)pq_i.w * p.ntypes;
         const int nty = p.ntypes;
-        const float l0 = rl[0], l1 = nty > 1 ? rl[1] : 0.0f, l2 = nty > 2 ? rl[2] : 0.0f, l3 = nty > 3 ? rl[3] : 0.0f;
+        const float mg = R.mg;  // (FP64 path: the words' margin)
+        const float l0 = rl[0] + mg, l1 = nty > 1 ? rl[1] + mg : 0.0f, l2 = nty > 2 ? rl[2] + mg : 0.0f,
+                    l3 = nty > 3 ? rl[3] + mg : 0.0f;
         const float lmax = fmaxf(fmaxf(l0, l1), fmaxf(l2, l3));
-        const uint32_t st_s = (uint32_t)__cvta_generic_to_shared(dyn);
+        const uint4* const st = st_u;  // (REL: FP32 coordinates in the first three words)
         // position inside the own cell (the binning of B1: cell = (u * nc) >> 32,
         // so the low word of u * nc is the fraction), for culling the rows and
         // row ends that lie wholly beyond the largest list radius of this
@@ -1379,10 +1411,10 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
         const float lcut = (sqrtf(lmax) + 1e-3f * wc) * (sqrtf(lmax) + 1e-3f * wc);  // rounding margin
         const int tsh = __ffs(T) - 1;
 #define KAMD_SCAN(R_, N_)                                                                                         \
-  scan_particle_mix<R_, N_>(st_s, s_ub, ncand, nc, nr, UX, UY, own_u, fxl, fyl, fzl, wc, lcut, sl, tsh, x, y, z, pq_i, \
+  scan_particle_mix<R_, N_>(st, s_ub, ncand, nc, nr, UX, UY, own_u, fxl, fyl, fzl, wc, lcut, sl, tsh, x, y, z, pq_i, \
                             sc, l0, l1, l2, l3, own_q, lb, gsz, p.maxrows, b1, b2, b3)
 #define KAMD_SCAN2(R_, N_)                                                                                           \
-  scan_particle_pair_mix<R_, N_>(st_s, s_ub, nr, UX, UY, own_u, fxl, fyl, fzl, wc, lcut, h,                         \
+  scan_particle_pair_mix<R_, N_>(st, s_ub, nr, UX, UY, own_u, fxl, fyl, fzl, wc, lcut, h,                         \
                                  3u << (threadIdx.x & 30u), x, y, z, pq_i, sc, l0, l1, l2, l3, own_q, lb, gsz,        \
                                  p.maxrows)
         if (pair) {
@@ -1399,43 +1431,6 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
 #undef KAMD_SCAN
 #undef KAMD_SCAN2
         if (sl == 0 && h == 0) p.xbq[i] = pq_i;
-      } else {
-        const double4_32a pi = p.p4[cur][i];
-        const int tb = (int)pi.w * p.ntypes;
-        const double L = R.L, hL = 0.5 * R.L;
-        double lmax = 0.0;
-        for (int t = 0; t < p.ntypes; ++t) lmax = fmax(lmax, sh.rl2d[tb + t]);
-        // position inside the own cell, for the same culling as the mixed path
-        const double wc = R.L / (double)(nc > 0 ? nc : 1);
-        const double fxl = pi.x - ccx * wc, fyl = pi.y - ccy * wc, fzl = pi.z - ccz * wc;
-        const double lcut = (sqrt(lmax) + 1e-9 * wc) * (sqrt(lmax) + 1e-9 * wc);
-        auto fd = [&](int o, double f) { return o < 0 ? f + (-o - 1) * wc : (o > 0 ? (wc - f) + (o - 1) * wc : 0.0); };
-        for (int run = 0; run < nruns; ++run) {
-          int qs = 0, qe = ncand;
-          if (nc > 0) {
-            const int oy = run % side - nr, oz = run / side - nr;
-            const double ey = fd(oy, fyl), ez = fd(oz, fzl);
-            const double d2 = ey * ey + ez * ez;
-            if (d2 >= lcut) continue;
-            int xl = -nr, xh = nr;
-            while (xl < 0 && fd(xl, fxl) * fd(xl, fxl) + d2 >= lcut) ++xl;
-            while (xh > 0 && fd(xh, fxl) * fd(xh, fxl) + d2 >= lcut) --xh;
-            const int us0 = ((lz + nr + oz) * UY + (ly + nr + oy)) * UX + lx + nr;
-            qs = s_ub[us0 + xl];
-            qe = s_ub[us0 + xh + 1];
-          }
-          for (int q = qs + sl; q < qe; q += T) {
-            const double4_32a pj = st_d[q];
-            double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-            if (dx > hL) dx -= L; else if (dx < -hL) dx += L;
-            if (dy > hL) dy -= L; else if (dy < -hL) dy += L;
-            if (dz > hL) dz -= L; else if (dz < -hL) dz += L;
-            if (q != own_q && dx * dx + dy * dy + dz * dz < sh.rl2d[tb + (int)pj.w]) {
-              list_push(lb, gsz, p.maxrows, k, b1, b2, b3, st_j[q]);
-            }
-          }
-        }
-        if (sl == 0) p.xbd[i] = pi;
       }
       if (!pair) list_flush(lb, gsz, p.maxrows, k, b1, b2, b3);
       if (h == 0) {
@@ -1460,7 +1455,7 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
     const RepDev& R = p.reps[p.tile_rep[i >> 5]];
     if (i - R.off >= R.n || !R.want_rebuild || R.nc == 0) continue;
     int cx, cy, cz;
-    cell_of_pos<MIX>(p, R, i, cur, cx, cy, cz);
+    cell_of_pos(p, R, i, cur, cx, cy, cz);
     const int c = (cz * R.nc + cy) * R.nc + cx;
     p.cellof[i] = c;
     atomicAdd(&p.ccount[R.cell0 + c], 1);
@@ -1638,6 +1633,7 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
             fo[cc] = p.frcd[cc * nt + o];
           }
           p.t_p4[d] = x;
+          p.pq[cur][d] = words_of(R.fx32, x.x, x.y, x.z, ty);
           for (int cc = 0; cc < 3; ++cc) {
             ((double*)p.t_vel)[cc * nt + d] = v[cc];
             ((double*)p.t_frc)[cc * nt + d] = fo[cc];
@@ -1690,15 +1686,10 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
     p.gid[i] = gd;
     p.typ[i] = ty;
   }
-  // mixed path: B5 and B6 share a phase (B6 reads only the gather copy,
-  // written in B4, and writes only the lists); FP64: B6 reads the positions
-  // that B5 moves back, so a barrier separates them
-  if constexpr (!MIX) {
-    f = grid_sync(p, sh, 105);
-    if (f < 0) return false;
-  }
+  // B5 and B6 share a phase: B6 reads only the gather copy, written in B4, and
+  // writes only the lists and their references
   // B6: Verlet lists (build_lists)
-  build_lists<MIX>(p, sh, cur);
+  build_lists(p, sh, cur);
   f = grid_sync(p, sh, 106);
   if (f < 0) return false;
   *fl = f;
@@ -1754,10 +1745,9 @@ __global__ void __launch_bounds__(512, KAMD_MIN_BLOCKS) md_persistent(KParams p)
     sh.vshf[t] = p.vsh_f[t];
     sh.rl2f[t] = p.rl2_f[t];
     sh.rli2f[t] = p.rli2_f[t];
+    sh.rcw2f[t] = p.rcw2_f[t];
     sh.tabd[t] = make_double4_32a(p.tab_d[t][0], p.tab_d[t][1], p.tab_d[t][2], p.tab_d[t][3]);
-    sh.vshd[t] = p.vsh_d[t];
-    sh.rl2d[t] = p.rl2_d[t];
-    sh.rli2d[t] = p.rli2_d[t];
+    sh.tabed[t] = make_double2(p.tabe_d[t][0], p.tabe_d[t][1]);
   }
   if (threadIdx.x < 8) sh.sm_bits[threadIdx.x] = 0u;
   if (threadIdx.x == 0) p.cta_sm[blockIdx.x] = sm_id();
@@ -1815,7 +1805,7 @@ __global__ void __launch_bounds__(512, KAMD_MIN_BLOCKS) md_persistent(KParams p)
       // follow, each closed by a grid barrier. Positions do not move, so each
       // build writes the same lists again.
       for (int64_t k = 1; k < p.nsteps; ++k) {
-        build_lists<MIX>(p, sh, cur);
+        build_lists(p, sh, cur);
         if ((fl = grid_sync(p, sh, 19)) < 0) return;
       }
       finish(false, fvalid);
