@@ -81,6 +81,22 @@ __device__ __forceinline__ uint4 words_of(double s, double x, double y, double z
                     (uint32_t)__double2loint(fma(z, s, big)), type);
 }
 
+// 1/x in FP64: the hardware's 20-bit estimate y and one step of the cubically
+// convergent iteration y (1 + e + e^2), e = 1 - x y: e^3 < 2^-60.
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// Minimum image of one coordinate difference (the branch rule; the comparison
+// is made on the bit patterns of non-negative doubles).
+__device__ __forceinline__ double image_f64(double d, double L, long long hLb) {
+  if ((__double_as_longlong(d) & 0x7fffffffffffffffll) > hLb) d -= copysign(L, d);
+  return d;
+}
+
 __device__ __forceinline__ double wrap_box(double x, double L) {
   x -= L * floor(x / L);
   if (x >= L) x -= L;

@@ -390,22 +390,6 @@ __device__ __forceinline__ void lane_sum_mix(const Shared& sh, const uint4* __re
   if (r > 2) pair_mix<ENERGY>(sh, pi, pq[jq.z], tb, sc, fx, fy, fz, pe, vir);
 }
 
-// 1/x in FP64: the hardware's 20-bit estimate y and one step of the cubically
-// convergent iteration y (1 + e + e^2), e = 1 - x y: e^3 < 2^-60.
-__device__ __forceinline__ double rcp_f64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
-// Minimum image of one coordinate difference (the branch rule; the comparison
-// is made on the bit patterns of non-negative doubles).
-__device__ __forceinline__ double image_f64(double d, double L, long long hLb) {
-  if ((__double_as_longlong(d) & 0x7fffffffffffffffll) > hLb) d -= copysign(L, d);
-  return d;
-}
-
 // Pair term for one list entry (FP64 path), Eq. (KAFix) and Eq. (VshiftedKALJ)
 // with sigma folded into the constants (16 FP64 operations without energy, 12
 // of them FMAs or multiplies of the pair itself).
