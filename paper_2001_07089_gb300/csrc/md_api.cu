@@ -22,6 +22,7 @@ struct md_system {
   bool mixed = true;
   std::vector<int64_t> n_per, out0;
   std::vector<double> L_per;
+  std::vector<int64_t> n_type0;  // particles of type 0 per replica
   double eps[16] = {0}, sig[16] = {0}, rc[16] = {0};
   double mass = 1.0;
   md_tuning tun{4, 256, 0.3, 0.7};
@@ -284,158 +285,285 @@ __global__ void k_unwrapped(bool mixed, int64_t ntot, const RepDev* reps, const 
   }
 }
 
-// Per-tile sums of squared displacement per type (Eq. (msdwithi)); counts in
-// the second half of the partial row.
-__global__ void k_msd_tiles(bool mixed, int ntiles, int ntypes, int64_t ntot, const RepDev* reps, const int32_t* tile_rep,
-                            const uint64_t* pfx, const double4_32a* p4, const int32_t* gid, const uint8_t* typ,
-                            const int32_t* img, const double* ref, double* part) {
-  const int lane = threadIdx.x & 31;
-  const int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (tile >= ntiles) return;
-  const RepDev& R = reps[tile_rep[tile]];
-  const int64_t i = tile * 32 + lane;
-  double d2 = 0.0;
-  int t = -1;
-  if (i - R.off < R.n) {
+// Sums of squared displacement per type (Eq. (msdwithi)), one record of sums
+// and counts per CTA: each thread adds up its particles, then warp trees and the
+// CTA's warps in order. The grid is fixed by the number of tiles, so the order
+// of every sum is too. (One record per tile, added up by a single thread, took
+// 3.5 ms at N = 10^6.)
+#define MSD_THREADS 256
+#define MSD_BLOCKS 1024
+__device__ __forceinline__ void msd_reduce(const double* v, const double* cnt, int ntypes, double* out) {
+  __shared__ double red[MSD_THREADS / 32][2 * MD_MAXTYPES];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int a = 0; a < ntypes; ++a) {
+    const double x = kamd::warp_sum(v[a]), y = kamd::warp_sum(cnt[a]);
+    if (lane == 0) {
+      red[warp][a] = x;
+      red[warp][MD_MAXTYPES + a] = y;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * MD_MAXTYPES && (threadIdx.x & (MD_MAXTYPES - 1)) < ntypes) {
+    double t = red[0][threadIdx.x];
+    for (int w = 1; w < MSD_THREADS / 32; ++w) t += red[w][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+}
+__global__ void __launch_bounds__(MSD_THREADS) k_msd_blocks(bool mixed, int ntypes, int64_t ntot, const RepDev* reps,
+                                                            const int32_t* tile_rep, const uint64_t* pfx,
+                                                            const double4_32a* p4, const int32_t* gid, const uint8_t* typ,
+                                                            const int32_t* img, const double* ref, double* part) {
+  double v[MD_MAXTYPES] = {0, 0, 0, 0};
+  double cnt[MD_MAXTYPES] = {0, 0, 0, 0};
+  int n[MD_MAXTYPES] = {0, 0, 0, 0};
+  for (int64_t i = (int64_t)blockIdx.x * MSD_THREADS + threadIdx.x; i < ntot; i += (int64_t)gridDim.x * MSD_THREADS) {
+    const RepDev& R = reps[tile_rep[i >> 5]];
+    if (i - R.off >= R.n) continue;
     const int64_t g = gid[i];
-    t = typ[i];
+    const int t = typ[i];
+    double d2 = 0.0;
     for (int c = 0; c < 3; ++c) {
       const double x = mixed ? kamd::from_fixed(pfx[c * ntot + i], R.L) : (c == 0 ? p4[i].x : c == 1 ? p4[i].y : p4[i].z);
       const double d = x + R.L * (double)img[c * ntot + i] - ref[3 * g + c];
       d2 += d * d;
     }
-  }
-  for (int a = 0; a < ntypes; ++a) {
-    const double v = kamd::warp_sum(t == a ? d2 : 0.0);
-    const double cnt = kamd::warp_sum(t == a ? 1.0 : 0.0);
-    if (lane == 0) {
-      part[tile * MD_NPART + a] = v;
-      part[tile * MD_NPART + MD_MAXTYPES + a] = cnt;
+#pragma unroll
+    for (int a = 0; a < MD_MAXTYPES; ++a) {
+      if (t == a) {
+        v[a] += d2;
+        ++n[a];
+      }
     }
   }
+#pragma unroll
+  for (int a = 0; a < MD_MAXTYPES; ++a) cnt[a] = (double)n[a];
+  msd_reduce(v, cnt, ntypes, part + (int64_t)blockIdx.x * 2 * MD_MAXTYPES);
 }
 
-// One thread per type: fixed-order sum over all tiles.
-__global__ void k_msd_final(int ntiles, int ntypes, const double* part, double* out) {
-  const int a = threadIdx.x;
-  if (a >= ntypes) return;
-  double s = 0.0, c = 0.0;
-  for (int t = 0; t < ntiles; ++t) {
-    s += part[(int64_t)t * MD_NPART + a];
-    c += part[(int64_t)t * MD_NPART + MD_MAXTYPES + a];
-  }
-  out[a] = c > 0 ? s / c : 0.0;
+// The blocks' records, strided over the threads of one CTA, then as above.
+__global__ void __launch_bounds__(MSD_THREADS) k_msd_final(int nblocks, int ntypes, const double* part, double* out) {
+  __shared__ double tot[2 * MD_MAXTYPES];
+  double v[MD_MAXTYPES] = {0, 0, 0, 0}, cnt[MD_MAXTYPES] = {0, 0, 0, 0};
+  for (int t = threadIdx.x; t < nblocks; t += MSD_THREADS)
+#pragma unroll
+    for (int a = 0; a < MD_MAXTYPES; ++a)
+      if (a < ntypes) {
+        v[a] += part[(int64_t)t * 2 * MD_MAXTYPES + a];
+        cnt[a] += part[(int64_t)t * 2 * MD_MAXTYPES + MD_MAXTYPES + a];
+      }
+  msd_reduce(v, cnt, ntypes, tot);
+  __syncthreads();
+  if (threadIdx.x < ntypes) out[threadIdx.x] = tot[MD_MAXTYPES + threadIdx.x] > 0 ? tot[threadIdx.x] / tot[MD_MAXTYPES + threadIdx.x] : 0.0;
 }
 
 // Pair-distance histogram of Sec. "Radial distribution function with
 // Python": every unordered pair with r < nbins*dr adds 2 (like) or 1 (unlike)
 // to bin floor(r/dr) of its replica (integer counts; exact, order-free).
-// Mixed path: a conservative FP32 test on the 32-bit gather words rejects the
-// pairs beyond r_max (most candidates); the bin of the others comes from the
-// exact 64-bit positions in FP64, as before. A block whose particles all
-// belong to one replica (and nbins <= RDF_SMEM_BINS) counts into a shared-
-// memory histogram and adds it to the replica's histogram once.
+//
+// A warp takes a unit, the particles of up to RDF_CELLS neighbouring cells of
+// one row, and the half of the rows around theirs that makes each pair of rows
+// meet once (of its own row, the slots after each particle's). Row members are
+// read 32 at a time, one per lane, straight from the gather copy, and tested in
+// FP32 against each particle of the unit; pairs within rmax (about one in ten)
+// wait in a queue until a full warp of them is binned. The bin follows from the
+// FP32 distance unless that lies within its own error of a bin edge; such pairs
+// (about one in a thousand at dr = 0.01) are binned from the exact positions in
+// FP64. So the counts are those of the exact distances, and GB300's slow FP64
+// unit, which computed every pair's difference, root and quotient before, has
+// next to nothing to do. Cells are those of the last list build; every particle
+// has moved less than half the outer skin since, so rows are reached out to
+// rmax + skin. A replica with too few cells for that is one row of all its slots.
+// Measured at N = 10^6, 400 bins to 4 sigma, with the MSD call: 30.6 ms -> 3.5 ms.
 #define RDF_SMEM_BINS 1024
-__global__ void k_rdf(bool mixed, int64_t ntot, int nbins, double dr, double skin, const RepDev* reps,
-                      const int32_t* tile_rep, int cur, const uint4* pq, const uint64_t* pfx, const double4_32a* p4,
-                      const uint8_t* typ, const int32_t* cstart, unsigned long long* hist) {
-  __shared__ unsigned int sh_h[3 * RDF_SMEM_BINS];
-  __shared__ int sh_rep;
-  const int64_t b0 = (int64_t)blockIdx.x * blockDim.x;
-  const int64_t i = b0 + threadIdx.x;
-  if (threadIdx.x == 0) {
-    const int64_t last = min(b0 + (int64_t)blockDim.x, ntot) - 1;
-    const int r0 = tile_rep[b0 >> 5];
-    sh_rep = (nbins <= RDF_SMEM_BINS && tile_rep[last >> 5] == r0) ? r0 : -1;
-  }
-  __syncthreads();
-  const bool priv = sh_rep >= 0;
-  if (priv)
-    for (int t = threadIdx.x; t < 3 * nbins; t += blockDim.x) sh_h[t] = 0u;
-  __syncthreads();
-  bool act = i < ntot;
-  const int r = act ? tile_rep[i >> 5] : 0;
-  const RepDev& R = reps[r];
-  if (act && i - R.off >= R.n) act = false;
-  if (act) {
-    const double rmax = dr * nbins, rmax2 = rmax * rmax;
-    const float rmax2f = (float)(rmax2 * (1.0 + 1e-4)) + 1e-6f;  // FP32 pre-test, widened
-    const float scf = R.fxs;
-    const int ti = typ[i];
-    double xi[3];
-    uint64_t ui[3];
-    for (int c = 0; c < 3; ++c) {
-      if (mixed) ui[c] = pfx[c * ntot + i];
-      else xi[c] = c == 0 ? p4[i].x : c == 1 ? p4[i].y : p4[i].z;
-    }
-    const uint4 qi = mixed ? pq[i] : make_uint4(0u, 0u, 0u, 0u);
-    const int nc = R.nc;
-    const int layers = nc > 0 ? (int)ceil((rmax + skin) * (1.0 + 1e-6) / (double)R.cellw) : 0;
-    const bool all = nc == 0 || 2 * layers + 1 > nc;
-    int cx = 0, cy = 0, cz = 0;
-    if (!all) {
-      if (mixed) {
-        cx = (int)(((uint64_t)(uint32_t)(ui[0] >> 32) * (uint64_t)nc) >> 32);
-        cy = (int)(((uint64_t)(uint32_t)(ui[1] >> 32) * (uint64_t)nc) >> 32);
-        cz = (int)(((uint64_t)(uint32_t)(ui[2] >> 32) * (uint64_t)nc) >> 32);
-      } else {
-        const double sc = (double)nc * R.invL;
-        cx = min(max((int)(xi[0] * sc), 0), nc - 1);
-        cy = min(max((int)(xi[1] * sc), 0), nc - 1);
-        cz = min(max((int)(xi[2] * sc), 0), nc - 1);
-      }
-    }
-    unsigned long long* h = hist + (int64_t)r * 3 * nbins;
-    auto visit = [&](int64_t j) {
-      if (j <= i) return;
-      if (mixed) {
-        const uint4 qj = pq[j];
-        const float fx = (float)(int)(qi.x - qj.x) * scf, fy = (float)(int)(qi.y - qj.y) * scf,
-                    fz = (float)(int)(qi.z - qj.z) * scf;
-        if (!(fmaf(fx, fx, fmaf(fy, fy, fz * fz)) < rmax2f)) return;
-      }
-      double d[3];
-      for (int c = 0; c < 3; ++c) {
-        if (mixed) {
-          d[c] = (double)(int64_t)(ui[c] - pfx[c * ntot + j]) * (R.L * (1.0 / 18446744073709551616.0));
-        } else {
-          const double xj = c == 0 ? p4[j].x : c == 1 ? p4[j].y : p4[j].z;
-          double e = xi[c] - xj;
-          if (e > 0.5 * R.L) e -= R.L;
-          else if (e < -0.5 * R.L) e += R.L;
-          d[c] = e;
-        }
-      }
-      const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-      if (!(r2 < rmax2)) return;
-      const int k = (int)(sqrt(r2) / dr);
-      if (k >= nbins) return;
-      const int tj = typ[j];
-      const int slot = (ti == 0 && tj == 0) ? k : ((ti == 1 && tj == 1) ? nbins + k : 2 * nbins + k);
-      const unsigned w = (ti == tj) ? 2u : 1u;
-      if (priv) atomicAdd(&sh_h[slot], w);
-      else atomicAdd(&h[slot], (unsigned long long)w);
-    };
-    if (all) {
-      for (int64_t j = R.off; j < R.off + R.n; ++j) visit(j);
-    } else {
-      // cells are those of the last list build; every particle has moved less
-      // than half a skin since, so layers computed with rmax + skin cover all pairs
-      for (int oz = -layers; oz <= layers; ++oz)
-        for (int oy = -layers; oy <= layers; ++oy)
-          for (int ox = -layers; ox <= layers; ++ox) {
-            const int c = (((cz + oz + 8 * nc) % nc) * nc + (cy + oy + 8 * nc) % nc) * nc + (cx + ox + 8 * nc) % nc;
-            const int lo = cstart[R.cs0 + c], hi = cstart[R.cs0 + c + 1];
-            for (int j = lo; j < hi; ++j) visit(j);
+#define RDF_CELLS 4
+#define RDF_PART 16  // particles of a unit that are tested in one go
+#define RDF_WARPS 8
+struct RdfArgs {
+  bool mixed;
+  int64_t ntot;
+  int nbins, blocks_per_rep;
+  double dr, skin;
+  const RepDev* reps;
+  const uint4* pq;
+  const uint64_t* pfx;
+  const double4_32a* p4;
+  const int32_t* cstart;
+  unsigned long long* hist;
+};
+struct RdfWarp {
+  float4 pos[RDF_PART];  // relative x, y, z, or words; the particle's type in w
+  float r2[64];          // queue: squared distance, the other's slot, particle of the unit | class << 8
+  int j[64];
+  int c[64];
+};
+
+template <bool REL>
+__device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfWarp& W, unsigned int* sh_h, bool priv, int r,
+                                         int i0, int np, uint4 ref, int lo, int n, bool own, float rmax2f, float invdr,
+                                         float edge, int& head, int& count) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const float sc = R.fxs;
+  auto bin = [&](int m) {  // the first m queued pairs
+    __syncwarp();
+    if (lane < m) {
+      const int q = (head + lane) & 63;
+      const float t = sqrtf(W.r2[q]) * invdr, fl = floorf(t);
+      const int cls = W.c[q] >> 8;
+      int k = (int)fl;
+      if (t - fl < edge || t - fl > 1.0f - edge) {
+        const int64_t i = i0 + (W.c[q] & 255), j = W.j[q];
+        const double rmax = a.dr * a.nbins;
+        double d[3];
+        for (int c = 0; c < 3; ++c) {
+          if (a.mixed) {
+            d[c] = (double)(int64_t)(a.pfx[c * a.ntot + i] - a.pfx[c * a.ntot + j]) * (R.L * (1.0 / 18446744073709551616.0));
+          } else {
+            const double xi = c == 0 ? a.p4[i].x : c == 1 ? a.p4[i].y : a.p4[i].z;
+            const double xj = c == 0 ? a.p4[j].x : c == 1 ? a.p4[j].y : a.p4[j].z;
+            double e = xi - xj;
+            if (e > 0.5 * R.L) e -= R.L;
+            else if (e < -0.5 * R.L) e += R.L;
+            d[c] = e;
           }
+        }
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        k = r2 < rmax * rmax ? (int)(sqrt(r2) / a.dr) : a.nbins;
+      }
+      if (k < a.nbins) {
+        const int slot = cls * a.nbins + k;
+        const unsigned w = cls < 2 ? 2u : 1u;
+        if (priv) atomicAdd(&sh_h[slot], w);
+        else atomicAdd(&a.hist[(int64_t)r * 3 * a.nbins + slot], (unsigned long long)w);
+      }
+    }
+    __syncwarp();
+    head += m;
+    count -= m;
+  };
+  if (lo < 0) {  // the unit is done: bin what waits
+    if (count > 0) bin(count);
+    return;
+  }
+  for (int t0 = 0; t0 < n; t0 += 32) {
+    const int j = lo + t0 + lane;
+    const bool in = t0 + lane < n;
+    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+    if (in) q = a.pq[j];
+    float x = 0.f, y = 0.f, z = 0.f;
+    if (REL) {
+      x = (float)(int)(q.x - ref.x) * sc;
+      y = (float)(int)(q.y - ref.y) * sc;
+      z = (float)(int)(q.z - ref.z) * sc;
+    }
+    for (int k = 0; k < np; ++k) {
+      const float4 P = W.pos[k];
+      float dx, dy, dz;
+      if (REL) {
+        dx = P.x - x;
+        dy = P.y - y;
+        dz = P.z - z;
+      } else {
+        dx = (float)(int)(__float_as_uint(P.x) - q.x) * sc;
+        dy = (float)(int)(__float_as_uint(P.y) - q.y) * sc;
+        dz = (float)(int)(__float_as_uint(P.z) - q.z) * sc;
+      }
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      const bool hit = in & (r2 < rmax2f) & (!own | (j > i0 + k));
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (m == 0u) continue;
+      if (hit) {
+        const int e = (head + count + __popc(m & below)) & 63;
+        const int ti = __float_as_int(P.w), tj = (int)q.w;
+        W.r2[e] = r2;
+        W.j[e] = j;
+        W.c[e] = k | ((ti == tj ? ti : 2) << 8);
+      }
+      count += __popc(m);
+      if (count >= 32) bin(32);
     }
   }
-  if (priv) {
-    __syncthreads();
-    unsigned long long* h = hist + (int64_t)sh_rep * 3 * nbins;
-    for (int t = threadIdx.x; t < 3 * nbins; t += blockDim.x)
-      if (sh_h[t]) atomicAdd(&h[t], (unsigned long long)sh_h[t]);
+}
+
+__global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
+  __shared__ unsigned int sh_h[3 * RDF_SMEM_BINS];
+  __shared__ RdfWarp sh_w[RDF_WARPS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = blockIdx.x / a.blocks_per_rep, b = blockIdx.x - r * a.blocks_per_rep;
+  const RepDev& R = a.reps[r];
+  const bool priv = a.nbins <= RDF_SMEM_BINS;
+  if (priv)
+    for (int t = threadIdx.x; t < 3 * a.nbins; t += blockDim.x) sh_h[t] = 0u;
+  __syncthreads();
+  const double rmax = a.dr * a.nbins, rmax2 = rmax * rmax;
+  const int nc = R.nc;
+  const int layers = nc > 0 ? (int)ceil((rmax + a.skin) * (1.0 + 1e-6) / (double)R.cellw) : 0;
+  const bool all = nc == 0 || 2 * layers + 1 > nc;
+  const int runs = all ? 0 : (nc + RDF_CELLS - 1) / RDF_CELLS;  // units per row of cells
+  const int units = all ? (R.n + RDF_PART - 1) / RDF_PART : runs * nc * nc;
+  const bool rel = !all && 2 * (RDF_CELLS + layers + 1) < nc;
+  // the FP32 distance is off by less than err: the rounding of coordinates of
+  // at most `span`, and the words' own error
+  const double span = rel ? (double)(RDF_CELLS + layers + 1) * (double)R.cellw : rmax;
+  const double err = 1e-6 * span + 8.0 * R.L / 4294967296.0;
+  const float edge = (float)(err / a.dr + 1e-6 * a.nbins), invdr = (float)(1.0 / a.dr);
+  const float rmax2f = (float)((rmax + 2.0 * err) * (rmax + 2.0 * err) * (1.0 + 1e-6));
+  RdfWarp& W = sh_w[warp];
+  for (int u = b * RDF_WARPS + warp; u < units; u += a.blocks_per_rep * RDF_WARPS) {
+    int s0, s1, x0 = 0, cy = 0, cz = 0, g = 0;
+    if (all) {
+      s0 = (int)R.off + u * RDF_PART;
+      s1 = min(s0 + RDF_PART, (int)R.off + R.n);
+    } else {
+      x0 = (u % runs) * RDF_CELLS;
+      cy = (u / runs) % nc;
+      cz = u / (runs * nc);
+      g = min(RDF_CELLS, nc - x0);
+      const int32_t* cs = a.cstart + R.cs0 + (cz * nc + cy) * nc + x0;
+      s0 = cs[0];
+      s1 = cs[g];
+    }
+    for (int i0 = s0; i0 < s1; i0 += RDF_PART) {
+      const int np = min(RDF_PART, s1 - i0);
+      const uint4 ref = a.pq[i0];
+      __syncwarp();
+      if (lane < np) {
+        const uint4 q = a.pq[i0 + lane];
+        const float t = __int_as_float((int)q.w);
+        W.pos[lane] = rel ? make_float4((float)(int)(q.x - ref.x) * R.fxs, (float)(int)(q.y - ref.y) * R.fxs,
+                                        (float)(int)(q.z - ref.z) * R.fxs, t)
+                          : make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), t);
+      }
+      __syncwarp();
+      int head = 0, count = 0;
+      auto scan = [&](int lo, int n, bool own) {
+        if (rel) rdf_scan<true>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
+        else rdf_scan<false>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
+      };
+      if (all) {
+        scan(i0, (int)R.off + R.n - i0, true);
+      } else {
+        const int len = min(2 * layers + g, nc);
+        const int a0 = len == nc ? 0 : (x0 - layers + nc) % nc;
+        const int over = max(a0 + len - nc, 0);
+        for (int oz = 0; oz <= layers; ++oz)
+          for (int oy = oz == 0 ? 0 : -layers; oy <= layers; ++oy) {
+            const int32_t* cs = a.cstart + R.cs0 + (((cz + oz) % nc) * nc + (cy + oy + nc) % nc) * nc;
+            // the run [a0, a0 + len) of cells, in two parts where it passes the box edge
+            for (int part = 0; part < (over > 0 ? 2 : 1); ++part) {
+              const int lo = cs[part ? 0 : a0], n = cs[part ? over : a0 + len - over] - lo;
+              if (n > 0) scan(lo, n, oz == 0 && oy == 0);
+            }
+          }
+      }
+      scan(-1, 0, false);
+    }
   }
+  if (!priv) return;
+  __syncthreads();
+  unsigned long long* h = a.hist + (int64_t)r * 3 * a.nbins;
+  for (int t = threadIdx.x; t < 3 * a.nbins; t += blockDim.x)
+    if (sh_h[t]) atomicAdd(&h[t], (unsigned long long)sh_h[t]);
 }
 
 // Pairs (i < j) inside their cutoff r < r_c,ab, from exact distances (mixed:
@@ -1198,7 +1326,12 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
     s->reps[r] = R;
     s->out0.push_back(o0);
     for (int t = 0; t < R.ntiles; ++t) tile_rep.push_back(r);
-    for (int64_t k = 0; k < n_per[r]; ++k) rep_of[o0 + k] = r;
+    int64_t n0 = 0;
+    for (int64_t k = 0; k < n_per[r]; ++k) {
+      rep_of[o0 + k] = r;
+      n0 += types[o0 + k] == 0;
+    }
+    s->n_type0.push_back(n0);
     off += (int64_t)R.ntiles * 32;
     o0 += n_per[r];
   }
@@ -1261,7 +1394,7 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
   AL(s->d_msd_ref[0], 3 * (size_t)ntotal);
   AL(s->d_io, 6 * (size_t)ntotal);
   AL(s->d_io_i, 3 * (size_t)ntotal);
-  AL(s->d_msd_part, (size_t)s->ntiles * MD_NPART);
+  AL(s->d_msd_part, (size_t)MSD_BLOCKS * 2 * MD_MAXTYPES);
   AL(s->d_count, 1);
 #undef AL
   s->stage_cap = stage_capacity(s);
@@ -1438,8 +1571,13 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
   for (int r = 0; r < s->nrep; ++r)
     if (dr * nbins > 0.5 * s->L_per[r] * (1 + 1e-12)) return fail(s, MD_ERR_INVALID_ARG, "nbins*dr must be <= L/2");
   if (reset || !s->d_rdf || nbins != s->rdf_nbins || dr != s->rdf_dr) {
-    dfree(s, s->d_rdf);
-    CKS(dalloc(s, &s->d_rdf, (size_t)s->nrep * 3 * nbins));
+    if (!s->d_rdf || nbins != s->rdf_nbins) {
+      dfree(s, s->d_rdf);
+      s->rdf_nbins = 0;
+      CKS(dalloc(s, &s->d_rdf, (size_t)s->nrep * 3 * nbins));
+    } else {
+      CK(cudaMemsetAsync(s->d_rdf, 0, 8 * (size_t)s->nrep * 3 * nbins, s->stream));
+    }
     s->rdf_nbins = nbins;
     s->rdf_dr = dr;
     s->rdf_meas = 0;
@@ -1448,22 +1586,34 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
   CKS(download_ctl(s));
   if (s->ctl.pending & MD_FLAG_REBUILD) CKS(run_op(s, MD_OP_REBUILD, MD_KIND_NVE, 0, 0, 0, 0, 0, 0, nullptr));
   CKS(download_ctl(s));
-  const int b = 128;
-  k_rdf<<<blocks_for(s->ntot, b), b, 0, s->stream>>>(s->mixed, s->ntot, (int)nbins, dr, s->tun.skin_outer, s->d_reps, s->d_tile_rep,
-                                                     s->ctl.cur, s->d_pq[s->ctl.cur], s->d_pfx, s->d_p4[s->ctl.cur],
-                                                     s->d_typ, s->d_cstart, s->d_rdf);
+  RdfArgs a;
+  a.mixed = s->mixed;
+  a.ntot = s->ntot;
+  a.nbins = (int)nbins;
+  a.dr = dr;
+  a.skin = s->tun.skin_outer;
+  a.reps = s->d_reps;
+  a.pq = s->d_pq[s->ctl.cur];
+  a.pfx = s->d_pfx;
+  a.p4 = s->d_p4[s->ctl.cur];
+  a.cstart = s->d_cstart;
+  a.hist = s->d_rdf;
+  // about eight CTAs per SM over all replicas, at most one warp per unit
+  // (a unit holds 8 particles or more in anything but a gas)
+  int64_t nmax = 0;
+  for (int64_t n : s->n_per) nmax = std::max(nmax, n);
+  a.blocks_per_rep = (int)std::max<int64_t>(
+      1, std::min<int64_t>((nmax / 8 + RDF_WARPS) / RDF_WARPS, (8 * (int64_t)s->nsm + s->nrep - 1) / s->nrep));
+  k_rdf<<<(unsigned)(a.blocks_per_rep * (int64_t)s->nrep), 32 * RDF_WARPS, 0, s->stream>>>(a);
   CK(cudaGetLastError());
   s->rdf_meas += 1;
   if (g) {
     std::vector<unsigned long long> h((size_t)s->nrep * 3 * nbins);
     CK(cudaMemcpyAsync(h.data(), s->d_rdf, 8 * h.size(), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    std::vector<uint8_t> types(s->n_total);
-    CK(cudaMemcpy(types.data(), s->d_typ_caller, s->n_total, cudaMemcpyDeviceToHost));
     for (int64_t k = 0; k < 3 * nbins; ++k) g[k] = 0.0;
     for (int r = 0; r < s->nrep; ++r) {
-      int64_t na = 0, nb = 0;
-      for (int64_t q = 0; q < s->n_per[r]; ++q) (types[s->out0[r] + q] == 0 ? na : nb) += 1;
+      const int64_t na = s->n_type0[r], nb = s->n_per[r] - na;
       // V and the shell volume of bin k; in two dimensions the area L^2 and the ring pi((k+1)^2 - k^2)dr^2
       const double Lr = s->L_per[r];
       const double V = s->ndim == 3 ? Lr * Lr * Lr : Lr * Lr;
@@ -1489,12 +1639,12 @@ md_status md_msd_tw(md_system* s, int slot, double* msd_per_type, int reset_refe
   CKS(download_ctl(s));
   if (reset_reference) CKS(reset_msd_ref(s, slot));
   if (!s->msd_valid[slot]) return fail(s, MD_ERR_INVALID_ARG, "MSD slot has no reference (reset it first)");
-  const int b = 256;
-  k_msd_tiles<<<blocks_for((int64_t)s->ntiles * 32, b), b, 0, s->stream>>>(
-      s->mixed, s->ntiles, s->ntypes, s->ntot, s->d_reps, s->d_tile_rep, s->d_pfx, s->d_p4[s->ctl.cur], s->d_gid,
-      s->d_typ, s->d_img, s->d_msd_ref[slot], s->d_msd_part);
+  const int nb = std::min(MSD_BLOCKS, (s->ntiles + MSD_THREADS / 32 - 1) / (MSD_THREADS / 32));
+  k_msd_blocks<<<nb, MSD_THREADS, 0, s->stream>>>(s->mixed, s->ntypes, s->ntot, s->d_reps, s->d_tile_rep, s->d_pfx,
+                                                  s->d_p4[s->ctl.cur], s->d_gid, s->d_typ, s->d_img,
+                                                  s->d_msd_ref[slot], s->d_msd_part);
   CK(cudaGetLastError());
-  k_msd_final<<<1, 32, 0, s->stream>>>(s->ntiles, s->ntypes, s->d_msd_part, s->d_io);
+  k_msd_final<<<1, MSD_THREADS, 0, s->stream>>>(nb, s->ntypes, s->d_msd_part, s->d_io);
   CK(cudaGetLastError());
   if (msd_per_type) CK(cudaMemcpyAsync(msd_per_type, s->d_io, 8 * s->ntypes, cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));

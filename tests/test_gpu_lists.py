@@ -1,0 +1,63 @@
+"""List builds and the FP64 force phase at the places where they can go wrong: entry queues that fill up
+before a list ends, and lists built inside a run (after force phases of the same launch)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2001_07089_gb300 import kamd
+from paper_2001_07089_gb300 import workloads as wl
+from tests.helpers import force_errors, melted
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kamd.load()
+
+
+@pytest.mark.parametrize("tpa", [1, 4, 8])
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("mixed", 1e-5)])
+def test_more_partners_than_a_queue_holds(prec, tol, tpa):
+    """One species with a cutoff of 4.5 in the melted N = 1000 liquid: about 460 partners per particle,
+    several times what the FP64 path's per-particle queues hold at once (128 or 256 entries)."""
+    pos, _, _, L = melted(1000, 22, nsteps=200)
+    types = np.zeros(1000, dtype=np.int32)
+    eps, sig, rc = np.array([[1.0]]), np.array([[0.9]]), np.array([[4.5]])
+    f_ref, v_ref, _ = oracle.forces(pos, types, oracle.Params(eps, sig, rc, 1.0), L)
+    with kamd.System(1000, L, types, eps, sig, rc, 1.0, 0.1, prec) as s:
+        s.set_tuning(threads_per_atom=tpa, skin=0.1, skin_outer=0.2)
+        s.set_state(pos)
+        f, pe, _ = s.forces()
+        entries = s.info()["list_entries"]
+    assert entries > 1000 * 400
+    emax, e2 = force_errors(f, f_ref)
+    assert emax <= tol and e2 <= tol, (emax, e2)
+    assert abs(pe[0] - v_ref) <= max(tol, 1e-6 if prec == "mixed" else 0) * abs(v_ref)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("tpa,block", [(1, 512), (4, 256), (8, 256)])
+def test_lists_built_in_a_run_equal_fresh_ones(prec, tpa, block):
+    """With a skin so small that every step rebuilds, the list of the last step belongs to the final
+    positions: a new system at those positions has as many candidate pairs, of either species."""
+    pos, vel, types, L = melted(1000, 24, nsteps=200)
+    counts = []
+    with kamd.System(1000, L, types, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec) as s:
+        s.set_tuning(threads_per_atom=tpa, block_size=block, skin=0.01, skin_outer=0.01)
+        s.set_state(pos, vel)
+        s.step_nve(0.005, 6)
+        info = s.info()
+        assert info["rebuilds"] >= 6
+        counts.append(info["list_entries"])
+        p, v, _ = s.get_state()
+    with kamd.System(1000, L, types, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec) as s:
+        s.set_tuning(threads_per_atom=tpa, block_size=block, skin=0.01, skin_outer=0.01)
+        s.set_state(p, v)
+        s.forces()
+        counts.append(s.info()["list_entries"])
+    # positions that pass through doubles may move a pair at the very edge of the radius
+    assert abs(counts[0] - counts[1]) <= 2, counts
