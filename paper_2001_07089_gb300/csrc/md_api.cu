@@ -66,14 +66,12 @@ struct md_system {
   int32_t* d_ccursor = nullptr;
   int32_t* d_chunk = nullptr;
   int32_t* d_cta_sm = nullptr;  // SM id per CTA of the persistent grid
-  int2* d_grp = nullptr;        // list-build groups (replica, index in replica)
   int2* d_redmap = nullptr;     // reduction chunks (replica, chunk index)
   int2* d_redrep = nullptr;     // per replica (first chunk, chunks)
   double* d_redpart = nullptr;  // chunk sums
   int64_t nred = 0;
   int red2 = 0;
   int red_tiles = MD_RED_TILES;
-  int64_t ngroups = 0;
   int cta_sm_cap = 0;
   int32_t* d_scat = nullptr;
   int32_t* d_nbr = nullptr;
@@ -495,7 +493,7 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   if (priv)
     for (int t = threadIdx.x; t < 3 * a.nbins; t += blockDim.x) sh_h[t] = 0u;
   __syncthreads();
-  const double rmax = a.dr * a.nbins, rmax2 = rmax * rmax;
+  const double rmax = a.dr * a.nbins;
   const int nc = R.nc;
   const int layers = nc > 0 ? (int)ceil((rmax + a.skin) * (1.0 + 1e-6) / (double)R.cellw) : 0;
   const bool all = nc == 0 || 2 * layers + 1 > nc;
@@ -766,6 +764,7 @@ void choose_groups(md_system* s) {
     R.gx = gx;
     R.gy = gy;
     R.gz = gz;
+    R.ngrp = R.nc > 0 ? ((R.nc + gx - 1) / gx) * ((R.nc + gy - 1) / gy) * ((R.nc + gz - 1) / gz) : 1;
   }
 }
 
@@ -828,15 +827,6 @@ md_status alloc_cells_and_list(md_system* s, int cap_entries) {
   CKS(dalloc(s, &s->d_ccursor, (size_t)s->ncells));
   CKS(dalloc(s, &s->d_chunk, (size_t)(s->ncells / MD_SCAN_CHUNK + 1)));
   {
-    std::vector<int2> grp;
-    for (int r = 0; r < s->nrep; ++r) {
-      const int nc = s->reps[r].nc;
-      if (nc == 0) continue;
-      const RepDev& R = s->reps[r];
-      const int ng = ((nc + R.gx - 1) / R.gx) * ((nc + R.gy - 1) / R.gy) * ((nc + R.gz - 1) / R.gz);
-      for (int k = 0; k < ng; ++k) grp.push_back(make_int2(r, k));
-    }
-    s->ngroups = (int64_t)grp.size();
     // two-level reductions (chunks of red_tiles tiles) once a replica spans
     // more than 4 chunks: below that, one CTA per replica is as fast and, in
     // NVE, its reduction overlaps the next step instead of adding a barrier.
@@ -871,13 +861,6 @@ md_status alloc_cells_and_list(md_system* s, int cap_entries) {
       CK(cudaMemcpyAsync(s->d_redmap, rmap.data(), sizeof(int2) * rmap.size(), cudaMemcpyHostToDevice, s->stream));
       CK(cudaMemcpyAsync(s->d_redrep, rrep.data(), sizeof(int2) * rrep.size(), cudaMemcpyHostToDevice, s->stream));
       CK(cudaStreamSynchronize(s->stream));  // local vectors
-    }
-    dfree(s, s->d_grp);
-    s->d_grp = nullptr;
-    CKS(dalloc(s, &s->d_grp, std::max<size_t>(grp.size(), 1)));
-    if (!grp.empty()) {
-      CK(cudaMemcpyAsync(s->d_grp, grp.data(), sizeof(int2) * grp.size(), cudaMemcpyHostToDevice, s->stream));
-      CK(cudaStreamSynchronize(s->stream));  // grp is a local vector
     }
   }
   const size_t entries = (size_t)s->ntiles * s->maxrows * 32 * T;
@@ -1000,8 +983,6 @@ KParams make_params(const md_system* s) {
   p.ccursor = s->d_ccursor;
   p.chunk = s->d_chunk;
   p.cta_sm = s->d_cta_sm;
-  p.grp = s->d_grp;
-  p.ngroups = s->ngroups;
   p.red2 = s->red2;
   p.red_tiles = s->red_tiles;
   p.nred = s->nred;
@@ -1962,7 +1943,7 @@ void md_destroy(md_system* s) {
   dfree(s, s->d_gid); dfree(s, s->d_typ); dfree(s, s->d_img);
   dfree(s, s->d_tpfx); dfree(s, s->d_tp4); dfree(s, s->d_tvel); dfree(s, s->d_tfrc); dfree(s, s->d_tgid); dfree(s, s->d_ttyp);
   dfree(s, s->d_timg);
-  dfree(s, s->d_cellof); dfree(s, s->d_cell_rep); dfree(s, s->d_ccount); dfree(s, s->d_cstart); dfree(s, s->d_ccursor); dfree(s, s->d_chunk); dfree(s, s->d_cta_sm); dfree(s, s->d_grp); dfree(s, s->d_redmap); dfree(s, s->d_redrep); dfree(s, s->d_redpart); dfree(s, s->d_scat);
+  dfree(s, s->d_cellof); dfree(s, s->d_cell_rep); dfree(s, s->d_ccount); dfree(s, s->d_cstart); dfree(s, s->d_ccursor); dfree(s, s->d_chunk); dfree(s, s->d_cta_sm); dfree(s, s->d_redmap); dfree(s, s->d_redrep); dfree(s, s->d_redpart); dfree(s, s->d_scat);
   dfree(s, s->d_nbr); dfree(s, s->d_nnb); dfree(s, s->d_part[0]); dfree(s, s->d_part[1]); dfree(s, s->d_plog); dfree(s, s->d_plog_rec);
   dfree(s, s->d_typ_caller); dfree(s, s->d_rep_of_caller); dfree(s, s->d_thermo); dfree(s, s->d_io);
   dfree(s, s->d_io_i); dfree(s, s->d_rdf); dfree(s, s->d_msd_part); dfree(s, s->d_count);

@@ -81,7 +81,10 @@ struct RepDev {
   int64_t rebuilds;
   int64_t prune_epoch;    // force step whose inner list must be pruned first (set by drifts)
   int64_t rebuild_epoch;  // force step before which the outer list was last rebuilt
-  int64_t cell_base;      // particles in the cells of earlier replicas that rebuild with this one
+  int32_t ngrp;           // list-build groups of the replica (without cells: one)
+  // totals over the earlier replicas that rebuild with this one: particles in
+  // cells, list-build groups, cells
+  int64_t cell_base, grp_base, sort_base;
   int64_t list_entries;
 };
 
@@ -97,6 +100,7 @@ struct CtlDev {
   int64_t step;         // global step counter
   int64_t steps_done;   // steps completed by the current/last launch
   int64_t prunes;       // prune passes since creation
+  int64_t grp_total, sort_total;  // list-build groups and cells of the replicas that rebuild now
   int err_where;        // phase id where a barrier timed out
   int pad;
 #ifdef KAMD_PHASE_TIMERS
@@ -192,14 +196,12 @@ struct KParams {
   int32_t* ccursor;
   int32_t* chunk;      // per-chunk cell-count sums of the cell scan (MD_SCAN_CHUNK cells each)
   int32_t* cta_sm;     // SM id of each CTA of the current launch
-  const int2* grp;     // list-build groups: (replica, group index inside the replica)
   int red2;            // 1: reductions in two levels (some replica has more than 4 chunks)
   int red_tiles;       // tiles per reduction chunk
   int64_t nred;        // reduction chunks over all replicas
   const int2* redmap;  // chunk -> (replica, chunk index inside the replica)
   const int2* redrep;  // replica -> (first chunk, number of chunks)
   double* redpart;     // chunk sums, MD_NPART doubles per chunk
-  int64_t ngroups;
   int32_t* scat;
   int32_t* nbr;        // outer list
   int32_t* nnb;

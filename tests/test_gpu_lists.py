@@ -61,3 +61,31 @@ def test_lists_built_in_a_run_equal_fresh_ones(prec, tpa, block):
         counts.append(s.info()["list_entries"])
     # positions that pass through doubles may move a pair at the very edge of the radius
     assert abs(counts[0] - counts[1]) <= 2, counts
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("block", [128, 512])
+def test_partial_rebuilds_of_more_replicas_than_threads(prec, block):
+    """Replicas with and without cells, cold and hot, so that some rebuild while their neighbours do not;
+    at block 128 there are more of them than a CTA has threads. Each is bitwise its stand-alone run."""
+    sizes, temps = [250, 1000, 300, 2000, 500], [0.05, 3.0, 1.0, 0.3, 0.05, 2.0, 0.6]
+    ns = [sizes[k % 5] for k in range(150)]
+    Ts = [temps[k % 7] for k in range(150)]
+    Ls = [wl.box_length(n) for n in ns]
+    types = [wl.ka_types(n, 5 + k).astype(np.int32) for k, n in enumerate(ns)]
+    tun = dict(threads_per_atom=4, block_size=block, skin=0.3, skin_outer=0.3)
+
+    def run(n, L, t, T):
+        with kamd.System(n, L, t, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec) as s:
+            s.set_tuning(**tun)
+            s.init_lattice(T, seed=9)
+            s.step_nve(0.004, 40)
+            return s.get_state(), s.info()["rebuilds"]
+
+    (p, v, img), rebuilds = run(ns, Ls, np.concatenate(types), Ts)
+    assert rebuilds < 150 * 40
+    off = np.concatenate([[0], np.cumsum(ns)])
+    for k in (0, 1, 2, 3, 4, 71, 126, 127, 128, 129, 148, 149):
+        (q, w, j), _ = run(ns[k], Ls[k], types[k], Ts[k])
+        at = slice(off[k], off[k + 1])
+        assert np.array_equal(q, p[at]) and np.array_equal(w, v[at]) and np.array_equal(j, img[at]), k
