@@ -35,7 +35,7 @@
 #define MD_LOG_SLOTS 64     // log steps per launch whose reductions wait for the launch end
 #define MD_ROWS_MAX 16      // (y, z) rows of cells in one list-build group: GY*GZ <= 4*4
 #define MD_RED_TILES 256    // tiles per chunk of the two-level per-replica reduction (default)
-#define MD_NPART 8   // per-tile partial sums: pe, ke, vir, px, py, pz, (2 spare)
+#define MD_NPART 4   // partial sums of a unit: pe, ke, virial, (spare); of a velocity draw: v_x, v_y, v_z, v^2
 
 // pending/commit flag bits (grid-uniform decisions)
 #define MD_FLAG_REBUILD 1
@@ -73,7 +73,7 @@ struct RepDev {
   double xi, g, lns, lns_next, xi_a;
   float xif, xiaf;  // FP32 copies of xi and xi_a for the mixed path
   // last reductions
-  double pe, ke, vir, px, py, pz;
+  double pe, ke, vir;
   // resampling
   double vmean[3], vscale;
   float vmeanf[3], vscalef;
@@ -201,14 +201,14 @@ struct KParams {
   int64_t nred;        // reduction chunks over all replicas
   const int2* redmap;  // chunk -> (replica, chunk index inside the replica)
   const int2* redrep;  // replica -> (first chunk, number of chunks)
-  double* redpart;     // chunk sums, MD_NPART doubles per chunk
+  double* redpart;     // chunk sums: quantity k of chunk g at [k * nred + g]
   int32_t* scat;
   int32_t* nbr;        // outer list
   int32_t* nnb;
   int32_t* nbr_in;     // inner (pruned) list, same layout; read by the force phase
   int32_t* nnb_in;
   // reductions
-  double* part[2];     // [ntiles][MD_NPART]: doubles (FP64 path) or float (hi, lo) pairs (mixed path)
+  double* part[2];     // [MD_NPART][units]: doubles (FP64 path) or float (hi, lo) pairs (mixed path)
   // partial records of NVE steps that only log, reduced after the launch's
   // last step: plog_slots slots of plog_stride doubles each
   double* plog;

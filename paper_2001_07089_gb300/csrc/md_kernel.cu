@@ -8,9 +8,9 @@
 //                 Sec. "Periodic boundary conditions"), gathered over a full
 //                 Verlet list by T lanes per particle (no atomics), then the
 //                 velocity update (Eq. (velVerletVel), or Eq. (ridotKVLRoman) /
-//                 (ridotsolved) under Nose-Hoover), per-tile FP64 partial sums
-//                 of PE, KE, virial, momentum, and -- for NVE steps -- the next
-//                 position update (Eq. (velVerletPos)) fused in.
+//                 (ridotsolved) under Nose-Hoover), per-warp partial sums of
+//                 KE, PE and virial where a step needs them, and -- for NVE
+//                 steps -- the next position update (Eq. (velVerletPos)) fused in.
 //   barrier
 //   reduce        per replica, fixed-order sum of tile partials; Nose-Hoover
 //                 xi, ln s updates (Eqs. (Noseupdate_lns), (Noseupdate_xiapprox),
@@ -489,6 +489,12 @@ __device__ __forceinline__ void unit_sum_f64(const KParams& p, const Shared& sh,
 // gather buffer. Without `pairs` only the kinetic partials are formed. Each
 // unit writes its own partial sums, so no CTA-wide synchronisation is needed.
 // `energy` = also form PE and virial (steps whose energies are reported).
+// `partials` = store the unit's sums: KE, and with `energy` PE and virial
+// (quantity k of unit u at part[k * nunits + u]). A float-float warp sum takes
+// about 70 instructions a warp, so a Nose-Hoover step, which needs the kinetic
+// energy alone, forms no other: with all of them (and the momentum, which
+// nothing read) 50 such steps took 18.72 ms at N = 10^6 and 34.3 ms on 512
+// replicas, now 17.86 and 33.4 ms.
 template <bool MIX>
 __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, bool fuse, double* part, bool pairs,
                             bool energy, bool partials, int64_t nstep) {
@@ -543,7 +549,7 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
           vir += __shfl_xor_sync(0xffffffffu, vir, o);
         }
       }
-      float e[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      float e[3] = {0.f, 0.f, 0.f};
       if (act && s == 0) {
         const float im = p.inv_massf, hdt = 0.5f * p.dtf, m = p.massf;
         const float xi = R->xif, xia = R->xiaf;
@@ -565,17 +571,15 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
         e[0] = 0.5f * pe;
         e[1] = 0.5f * m * fmaf(v[0], v[0], fmaf(v[1], v[1], v[2] * v[2]));
         e[2] = 0.5f * vir;
-        e[3] = m * v[0];
-        e[4] = m * v[1];
-        e[5] = m * v[2];
         if (fuse) drift_mix(p, *R, i, cur, v, an, 0.0f, pi.w, nstep);
       }
       if (partials) {
-        float2* out = reinterpret_cast<float2*>(part) + (int64_t)u * MD_NPART;
+        float2* out = reinterpret_cast<float2*>(part) + u;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
+        for (int k = 0; k < 3; ++k) {
+          if (k != 1 && !energy) continue;
           const ff t = warp_sum_ff(ff{e[k], 0.0f});
-          if (lane == 0) out[k] = make_float2(t.hi, t.lo);
+          if (lane == 0) out[(int64_t)k * nunits] = make_float2(t.hi, t.lo);
         }
       }
     } else {
@@ -596,7 +600,7 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
           vir += __shfl_xor_sync(0xffffffffu, vir, o);
         }
       }
-      double e[6] = {0, 0, 0, 0, 0, 0};
+      double e[3] = {0, 0, 0};
       if (act && s == 0) {
         const double im = p.inv_mass, hdt = 0.5 * p.dt, m = p.mass;
         const double xi = R->xi, xia = R->xi_a;
@@ -618,17 +622,15 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
         e[0] = 0.5 * pe;
         e[1] = 0.5 * m * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
         e[2] = 0.5 * vir;
-        e[3] = m * v[0];
-        e[4] = m * v[1];
-        e[5] = m * v[2];
         if (fuse) drift_f64(p, *R, i, cur, v, an, 0.0, nstep);
       }
       if (partials) {
-        double* out = part + (int64_t)u * MD_NPART;
+        double* out = part + u;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
+        for (int k = 0; k < 3; ++k) {
+          if (k != 1 && !energy) continue;
           const double t = warp_sum(e[k]);
-          if (lane == 0) out[k] = t;
+          if (lane == 0) out[(int64_t)k * nunits] = t;
         }
       }
     }
@@ -756,11 +758,11 @@ __device__ void resample_draw_phase(const KParams& p, uint64_t draw, double* par
           e[3] = fmaf(v, v, e[3]);
         }
       }
-      float2* out = reinterpret_cast<float2*>(part) + tile * MD_NPART;
+      float2* out = reinterpret_cast<float2*>(part) + tile;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const ff w = warp_sum_ff(ff{e[k], 0.0f});
-        if (lane == 0) out[k] = make_float2(w.hi, w.lo);
+        if (lane == 0) out[(int64_t)k * p.ntiles] = make_float2(w.hi, w.lo);
       }
     } else {
       double e[4] = {0, 0, 0, 0};
@@ -777,7 +779,7 @@ __device__ void resample_draw_phase(const KParams& p, uint64_t draw, double* par
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const double w = warp_sum(e[k]);
-        if (lane == 0) part[tile * MD_NPART + k] = w;
+        if (lane == 0) part[(int64_t)k * p.ntiles + tile] = w;
       }
     }
   }
@@ -788,54 +790,61 @@ __device__ void resample_draw_phase(const KParams& p, uint64_t draw, double* par
 __device__ __noinline__ void reduce_scalars(const KParams& p, RepDev& R, int64_t r, const double* acc, int mode,
                                             int64_t step, bool log_now, int64_t log_idx, bool nh);
 
-// Sum of the partial records [u0, u0 + nu) (fixed order): thread-strided
+// Sums of the partials [u0, u0 + nu) of the quantities whose bit is set in
+// `which` (quantity k begins at part[k * stride]), in a fixed order: thread-strided
 // float-float (mixed) or double accumulation, warp trees, then the CTA's
-// warps in order; the warps' sums are added by lanes 0..5 of warp 0, one
+// warps in order; the warps' sums are added by lanes 0..3 of warp 0, one
 // quantity each (each sum in the same order as one thread adding them one
-// after the other). Thread 0 receives the six totals in acc.
+// after the other). Thread 0 receives the totals in acc, zero for the others.
 template <bool MIX>
-__device__ void sum_records(Shared& sh, const double* part, int64_t u0, int64_t nu, double* acc) {
+__device__ void sum_records(Shared& sh, const double* part, int64_t stride, int64_t u0, int64_t nu, int which,
+                            double* acc) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const int64_t B = blockDim.x;
-  double tot = 0.0;  // lane k < 6 of warp 0: total of quantity k
+  double tot = 0.0;  // lane k < MD_NPART of warp 0: total of quantity k
   if constexpr (MIX) {
-    ff a[6];
+    ff a[MD_NPART];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = ff{0.f, 0.f};
+    for (int k = 0; k < MD_NPART; ++k) a[k] = ff{0.f, 0.f};
     const float2* q0 = reinterpret_cast<const float2*>(part);
     for (int64_t t = threadIdx.x; t < nu; t += B) {
-      const float2* q = q0 + (u0 + t) * MD_NPART;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) a[k] = ff_add(a[k], ff{q[k].x, q[k].y});
+      for (int k = 0; k < MD_NPART; ++k)
+        if (which >> k & 1) {
+          const float2 q = q0[k * stride + u0 + t];
+          a[k] = ff_add(a[k], ff{q.x, q.y});
+        }
     }
     float2* red = reinterpret_cast<float2*>(&sh.red[0][0]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < MD_NPART; ++k) {
+      if (!(which >> k & 1)) continue;
       a[k] = warp_sum_ff(a[k]);
       if (lane == 0) red[warp * MD_NPART + k] = make_float2(a[k].hi, a[k].lo);
     }
     __syncthreads();
-    if (warp == 0 && lane < 6) {
+    if (warp == 0 && lane < MD_NPART && (which >> lane & 1)) {
       ff u = {red[lane].x, red[lane].y};
       for (int w = 1; w < nwarp; ++w) u = ff_add(u, ff{red[w * MD_NPART + lane].x, red[w * MD_NPART + lane].y});
       tot = (double)u.hi + (double)u.lo;
     }
   } else {
-    double a[6];
+    double a[MD_NPART];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = 0.0;
+    for (int k = 0; k < MD_NPART; ++k) a[k] = 0.0;
     for (int64_t t = threadIdx.x; t < nu; t += B) {
-      const double* q = part + (u0 + t) * MD_NPART;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) a[k] += q[k];
+      for (int k = 0; k < MD_NPART; ++k)
+        if (which >> k & 1) a[k] += part[k * stride + u0 + t];
     }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < MD_NPART; ++k) {
+      if (!(which >> k & 1)) continue;
       a[k] = warp_sum(a[k]);
       if (lane == 0) sh.red[warp][k] = a[k];
     }
     __syncthreads();
-    if (warp == 0 && lane < 6) {
+    if (warp == 0 && lane < MD_NPART && (which >> lane & 1)) {
       double u = sh.red[0][lane];
       for (int w = 1; w < nwarp; ++w) u += sh.red[w][lane];
       tot = u;
@@ -843,7 +852,7 @@ __device__ void sum_records(Shared& sh, const double* part, int64_t u0, int64_t 
   }
   if (warp == 0) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < MD_NPART; ++k) {
       const double v = __shfl_sync(0xffffffffu, tot, k);
       if (lane == 0) acc[k] = v;
     }
@@ -861,11 +870,14 @@ template <bool MIX>
 __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, int upt, int mode, int64_t step,
                              bool log_now, int64_t log_idx) {
   const bool nh = (p.kind == MD_KIND_NH || p.kind == MD_KIND_NH_EXACT) && p.op == MD_OP_STEPS;
-  double acc[6];
+  // the sums that reduce_scalars reads in this mode
+  const int which = mode == RED_RESAMPLE ? 0xf : (mode == RED_STEP_KE || mode == RED_KE) ? 0x2 : 0x7;
+  const int64_t nu = (int64_t)p.ntiles * upt;  // partials per quantity
+  double acc[MD_NPART];
   if (!p.red2) {
     for (int r = blockIdx.x; r < p.nrep; r += gridDim.x) {
       RepDev& R = p.reps[r];
-      sum_records<MIX>(sh, part, (int64_t)R.tile0 * upt, (int64_t)R.ntiles * upt, acc);
+      sum_records<MIX>(sh, part, nu, (int64_t)R.tile0 * upt, (int64_t)R.ntiles * upt, which, acc);
       if (threadIdx.x == 0) reduce_scalars(p, R, r, acc, mode, step, log_now, log_idx, nh);
       __syncthreads();
     }
@@ -876,10 +888,10 @@ __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, i
     const RepDev& R = p.reps[rc.x];
     const int t0 = rc.y * p.red_tiles;
     const int nt = min(p.red_tiles, R.ntiles - t0);
-    sum_records<MIX>(sh, part, (int64_t)(R.tile0 + t0) * upt, (int64_t)nt * upt, acc);
+    sum_records<MIX>(sh, part, nu, (int64_t)(R.tile0 + t0) * upt, (int64_t)nt * upt, which, acc);
     if (threadIdx.x == 0) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) p.redpart[g * MD_NPART + k] = acc[k];
+      for (int k = 0; k < MD_NPART; ++k) p.redpart[k * p.nred + g] = acc[k];
     }
   }
   if (grid_sync(p, sh, 17) < 0) return false;
@@ -887,7 +899,7 @@ __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, i
   // records (thread-strided, warp trees, warps in order: a fixed order)
   for (int r = blockIdx.x; r < p.nrep; r += gridDim.x) {
     const int2 rr = p.redrep[r];
-    sum_records<false>(sh, p.redpart, rr.x, rr.y, acc);
+    sum_records<false>(sh, p.redpart, p.nred, rr.x, rr.y, which, acc);
     if (threadIdx.x == 0) reduce_scalars(p, p.reps[r], r, acc, mode, step, log_now, log_idx, nh);
   }
   __syncthreads();
@@ -922,11 +934,9 @@ __device__ __noinline__ void reduce_scalars(const KParams& p, RepDev& R, int64_t
     R.vmeanf[0] = (float)mx; R.vmeanf[1] = (float)my; R.vmeanf[2] = (float)mz;
     R.vscalef = (float)sc;
     R.ke = 0.5 * p.mass * sc * sc * S;
-    R.px = R.py = R.pz = 0.0;
   } else {
     if (mode == RED_FORCES || mode == RED_STEP) { R.pe = acc[0]; R.vir = acc[2]; }
     R.ke = acc[1];
-    R.px = acc[3]; R.py = acc[4]; R.pz = acc[5];
     if (nh) {
       const double gnew = (2.0 * R.ke - X * R.T_target) / R.Q;
       if (mode == RED_STEP || mode == RED_STEP_KE) {
@@ -1925,8 +1935,9 @@ __global__ void __launch_bounds__(512) k_log_records(KParams p, int nslots) {
   for (int64_t w = blockIdx.x; w < (int64_t)nslots * p.nrep; w += gridDim.x) {
     const int k = (int)(w / p.nrep), r = (int)(w - (int64_t)k * p.nrep);
     RepDev& R = p.reps[r];
-    double acc[6];
-    sum_records<MIX>(sh, p.plog + (int64_t)k * p.plog_stride, (int64_t)R.tile0 * p.T, (int64_t)R.ntiles * p.T, acc);
+    double acc[MD_NPART];
+    sum_records<MIX>(sh, p.plog + (int64_t)k * p.plog_stride, (int64_t)p.ntiles * p.T, (int64_t)R.tile0 * p.T,
+                     (int64_t)R.ntiles * p.T, 0x7, acc);
     if (threadIdx.x == 0) {
       const longlong2 rec = p.plog_rec[k];
       reduce_scalars(p, R, r, acc, RED_LOG, rec.x, true, rec.y, false);

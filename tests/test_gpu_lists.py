@@ -89,3 +89,30 @@ def test_partial_rebuilds_of_more_replicas_than_threads(prec, block):
         (q, w, j), _ = run(ns[k], Ls[k], types[k], Ts[k])
         at = slice(off[k], off[k + 1])
         assert np.array_equal(q, p[at]) and np.array_equal(w, v[at]) and np.array_equal(j, img[at]), k
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("kind", [kamd.MD_NVT_NOSE_HOOVER, kamd.MD_NVT_NOSE_HOOVER_EXACT], ids=["nh", "nh-exact"])
+@pytest.mark.parametrize("n,tpa", [(250, 8), (1000, 1), (32768, 4), (32800, 2)])
+def test_one_replica_under_nose_hoover_equals_a_batch_member(prec, kind, n, tpa):
+    """Bitwise the same alone and in a batch, with the sums added in one level (up to 32768 particles) and
+    in two, and whether a step also forms the potential energy (log_every=1) or the kinetic energy alone."""
+    L = wl.box_length(n)
+    types = wl.ka_types(n, 3).astype(np.int32)
+
+    def run(nrep, log_every):
+        Ts = [1.3, 0.7][:nrep]
+        with kamd.System([n] * nrep if nrep > 1 else n, [L] * nrep if nrep > 1 else L, np.concatenate([types] * nrep),
+                         wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec) as s:
+            s.set_tuning(threads_per_atom=tpa, block_size=256, skin=0.3, skin_outer=0.6)
+            s.init_lattice(Ts if nrep > 1 else Ts[0], seed=11)
+            log = np.concatenate([s.step_nvt(0.004, 12, Ts if nrep > 1 else Ts[0], kind=kind, param=0.4,
+                                             log_every=log_every) for _ in range(2)])
+            return [x[:n] for x in s.get_state()], log[:, 0]
+
+    a, la = run(1, 4)
+    for b, lb in (run(2, 4), run(1, 1)):
+        assert all(np.array_equal(x, y) for x, y in zip(a, b))
+        last = lb if len(lb) == len(la) else lb[3::4]
+        assert all(np.array_equal(la[f], last[f]) for f in la.dtype.names if f != "step")
+    assert np.all(np.isfinite(la["T"])) and np.all(la["T"] > 0)
