@@ -15,7 +15,8 @@
 //   reduce        per replica, fixed-order sum of tile partials; Nose-Hoover
 //                 xi, ln s updates (Eqs. (Noseupdate_lns), (Noseupdate_xiapprox),
 //                 (FoxAndersen_ydottplush)); thermo record.
-//   [Nose-Hoover: barrier, position update Eq. (Noseupdate_ri), barrier]
+//   [Nose-Hoover: barrier (several replicas only), position update
+//    Eq. (Noseupdate_ri), barrier]
 //   [resampling step: Maxwell-Boltzmann draw, reduce, centre+rescale+drift]
 //   [rebuild when any particle moved > skin/2: cell count, scan, scatter,
 //    in-cell rank sort by caller index, permute, Verlet-list build]
@@ -45,6 +46,7 @@ struct Shared {
   double2 tabed[MD_MAXTYPES * MD_MAXTYPES];
   double red[16][MD_NPART];
   int scan[32];
+  RepDev lone;  // Nose-Hoover steps of a single replica: this CTA's copy (see reduce_phase)
   int snap;
   unsigned gen;  // grid barrier generation this CTA waits for next (thread 0)
   // SM-local work layout of this launch (see sm_layout)
@@ -289,8 +291,10 @@ __device__ __forceinline__ void drift_f64(const KParams& p, const RepDev& R, int
 // Stand-alone position update for every particle (first step of a call,
 // Nose-Hoover steps, and the step after a resampling). With `rescale` the
 // velocities are first centred and scaled by the replica's resampling factors.
+// `lone`: where a single replica's Nose-Hoover variables are (see reduce_phase).
 template <bool MIX>
-__device__ void drift_phase(const KParams& p, int cur, bool nh, bool rescale, bool drift, int64_t nstep) {
+__device__ void drift_phase(const KParams& p, int cur, bool nh, bool rescale, bool drift, int64_t nstep,
+                            const RepDev* lone = nullptr) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t nt = p.ntot;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += stride) {
@@ -310,7 +314,7 @@ __device__ void drift_phase(const KParams& p, int cur, bool nh, bool rescale, bo
           p.velf[c * nt + i] = v[c];
         }
       }
-      if (drift) drift_mix(p, R, i, cur, v, a, nh ? R.xif : 0.0f, p.pq[cur][i].w, nstep);
+      if (drift) drift_mix(p, R, i, cur, v, a, nh ? (lone ? lone->xif : R.xif) : 0.0f, p.pq[cur][i].w, nstep);
     } else {
       double v[3], a[3];
 #pragma unroll
@@ -325,7 +329,7 @@ __device__ void drift_phase(const KParams& p, int cur, bool nh, bool rescale, bo
           p.veld[c * nt + i] = v[c];
         }
       }
-      if (drift) drift_f64(p, R, i, cur, v, a, nh ? R.xi : 0.0, nstep);
+      if (drift) drift_f64(p, R, i, cur, v, a, nh ? (lone ? lone->xi : R.xi) : 0.0, nstep);
     }
   }
 }
@@ -530,6 +534,7 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
       int4 jq0 = make_int4(0, 0, 0, 0);
       if (cnt0 > 0) jq0 = __ldcs(reinterpret_cast<const int4*>(lp));
       const RepDev* R = &p.reps[p.tile_rep[tile]];
+      const RepDev* bath = (p.nrep == 1 && kick >= KICK_NH) ? &sh.lone : R;
       const bool act = (tile - R->tile0) * 32 + a < R->n;
       const int cnt = act ? cnt0 : 0;
       float fx = 0.f, fy = 0.f, fz = 0.f, pe = 0.f, vir = 0.f;
@@ -552,7 +557,7 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
       float e[3] = {0.f, 0.f, 0.f};
       if (act && s == 0) {
         const float im = p.inv_massf, hdt = 0.5f * p.dtf, m = p.massf;
-        const float xi = R->xif, xia = R->xiaf;
+        const float xi = bath->xif, xia = bath->xiaf;
         const float F[3] = {fx, fy, fz};
         float an[3];
 #pragma unroll
@@ -603,7 +608,8 @@ __device__ void force_phase(const KParams& p, Shared& sh, int cur, int kick, boo
       double e[3] = {0, 0, 0};
       if (act && s == 0) {
         const double im = p.inv_mass, hdt = 0.5 * p.dt, m = p.mass;
-        const double xi = R->xi, xia = R->xi_a;
+        const RepDev* bath = (p.nrep == 1 && kick >= KICK_NH) ? &sh.lone : R;
+        const double xi = bath->xi, xia = bath->xi_a;
         const double F[3] = {fx, fy, fz};
         double v[3], an[3];
 #pragma unroll
@@ -866,14 +872,53 @@ __device__ void sum_records(Shared& sh, const double* part, int64_t stride, int6
 // by separate CTAs, then, after a grid barrier, one CTA per replica adds its
 // chunk sums in chunk order. Both orders are fixed, so results are
 // reproducible. Returns false after a barrier timeout.
+// `lone` (Nose-Hoover steps of a single replica): every CTA adds the last level
+// itself, in the same order, and keeps its own copy of the replica's bath
+// variables in sh.lone, so no barrier stands between the sums and the position
+// update that needs them; CTA 0 also writes the replica. What bounds small
+// systems is the barriers (about 2 us each with the phase's latency): 50
+// steps of 1000 particles in a plane 1046 -> 931 us, of N = 10^6 17.86 ->
+// 17.70 ms. At 304 CTAs the repeated reads are 20 MB from L2 at most (the
+// largest system reduced in one level). With several replicas a CTA's
+// particles belong to many of them, and the barrier stays.
 template <bool MIX>
 __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, int upt, int mode, int64_t step,
-                             bool log_now, int64_t log_idx) {
+                             bool log_now, int64_t log_idx, bool lone = false) {
   const bool nh = (p.kind == MD_KIND_NH || p.kind == MD_KIND_NH_EXACT) && p.op == MD_OP_STEPS;
   // the sums that reduce_scalars reads in this mode
   const int which = mode == RED_RESAMPLE ? 0xf : (mode == RED_STEP_KE || mode == RED_KE) ? 0x2 : 0x7;
   const int64_t nu = (int64_t)p.ntiles * upt;  // partials per quantity
   double acc[MD_NPART];
+  if (p.red2) {
+    for (int64_t g = blockIdx.x; g < p.nred; g += gridDim.x) {
+      const int2 rc = p.redmap[g];
+      const RepDev& R = p.reps[rc.x];
+      const int t0 = rc.y * p.red_tiles;
+      const int nt = min(p.red_tiles, R.ntiles - t0);
+      sum_records<MIX>(sh, part, nu, (int64_t)(R.tile0 + t0) * upt, (int64_t)nt * upt, which, acc);
+      if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < MD_NPART; ++k) p.redpart[k * p.nred + g] = acc[k];
+      }
+    }
+    if (grid_sync(p, sh, 17) < 0) return false;
+  }
+  if (lone) {
+    if (p.red2) sum_records<false>(sh, p.redpart, p.nred, 0, p.nred, which, acc);
+    else sum_records<MIX>(sh, part, nu, 0, nu, which, acc);
+    if (threadIdx.x == 0) {
+      reduce_scalars(p, sh.lone, 0, acc, mode, step, log_now && blockIdx.x == 0, log_idx, true);
+      if (blockIdx.x == 0) {
+        RepDev& R = p.reps[0];
+        R.pe = sh.lone.pe; R.ke = sh.lone.ke; R.vir = sh.lone.vir;
+        R.xi = sh.lone.xi; R.g = sh.lone.g; R.xi_a = sh.lone.xi_a;
+        R.lns = sh.lone.lns; R.lns_next = sh.lone.lns_next;
+        R.xif = sh.lone.xif; R.xiaf = sh.lone.xiaf;
+      }
+    }
+    __syncthreads();
+    return true;
+  }
   if (!p.red2) {
     for (int r = blockIdx.x; r < p.nrep; r += gridDim.x) {
       RepDev& R = p.reps[r];
@@ -883,18 +928,6 @@ __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, i
     }
     return true;
   }
-  for (int64_t g = blockIdx.x; g < p.nred; g += gridDim.x) {
-    const int2 rc = p.redmap[g];
-    const RepDev& R = p.reps[rc.x];
-    const int t0 = rc.y * p.red_tiles;
-    const int nt = min(p.red_tiles, R.ntiles - t0);
-    sum_records<MIX>(sh, part, nu, (int64_t)(R.tile0 + t0) * upt, (int64_t)nt * upt, which, acc);
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int k = 0; k < MD_NPART; ++k) p.redpart[k * p.nred + g] = acc[k];
-    }
-  }
-  if (grid_sync(p, sh, 17) < 0) return false;
   // level 2: one CTA per replica sums the replica's chunk sums as FP64
   // records (thread-strided, warp trees, warps in order: a fixed order)
   for (int r = blockIdx.x; r < p.nrep; r += gridDim.x) {
@@ -1860,6 +1893,11 @@ __global__ void __launch_bounds__(512, KAMD_MIN_BLOCKS) md_persistent(KParams p)
     now_drifted = true;
     if ((fl = grid_sync(p, sh, 6)) < 0) return;
   }
+  const bool lone = nh && p.nrep == 1;
+  if (lone) {
+    if (threadIdx.x == 0) sh.lone = p.reps[0];
+    __syncthreads();
+  }
   for (int64_t s = 0; s < p.nsteps; ++s) {
     if (fl & MD_FLAG_UNSTABLE) break;
     const int64_t step = step0 + s + 1;
@@ -1893,13 +1931,14 @@ __global__ void __launch_bounds__(512, KAMD_MIN_BLOCKS) md_persistent(KParams p)
       if (blockIdx.x == 0 && threadIdx.x == 0) p.plog_rec[ndef] = make_longlong2(step, lidx);
       ++ndef;
     } else if (need_red &&
-               !reduce_phase<MIX>(p, sh, part, p.T, energy ? RED_STEP : RED_STEP_KE, step, log_now && !rs, lidx)) {
+               !reduce_phase<MIX>(p, sh, part, p.T, energy ? RED_STEP : RED_STEP_KE, step, log_now && !rs, lidx,
+                                  lone)) {
       return;
     }
     if (nh) {
-      if ((fl = grid_sync(p, sh, 11)) < 0) return;
+      if (!lone && (fl = grid_sync(p, sh, 11)) < 0) return;
       if (!last) {
-        drift_phase<MIX>(p, cur, true, false, true, step + 1);
+        drift_phase<MIX>(p, cur, true, false, true, step + 1, lone ? &sh.lone : nullptr);
         cur ^= 1;
         now_drifted = true;
         if ((fl = grid_sync(p, sh, 12)) < 0) return;
