@@ -116,6 +116,7 @@ struct md_system {
   cudaGraphNode_t gnode = nullptr;
   int g_grid = 0, g_block = 0;
   size_t g_smem = 0;
+  int carveout = 0, g_carveout = 0;  // percent of the SM's shared memory that the grid takes
   int64_t graph_launches = 0;
   int64_t kernel_launches = 0;  // persistent launches and log-record launches
   std::string err;
@@ -925,6 +926,12 @@ md_status configure_grid(md_system* s) {
   for (const auto& R : s->reps) groups = std::max(groups, R.ngrp);
   const bool small = groups <= s->nsm && (int64_t)s->ntiles * list_lanes(s) <= (int64_t)s->nsm * (b / 32);
   s->grid = (small ? 1 : per_sm) * s->nsm;
+  // The split between shared memory and L1 is asked for at each launch: no more
+  // shared memory than the resident CTAs take, since the force phase's gathers
+  // live in L1. The driver's own choice was larger: N = 10^6, force phase 199 ->
+  // 191 us; 20 steps of N = 8*10^6 56.3 -> 54.0 ms. (A launch attribute: other
+  // systems of the process have other needs.)
+  CK(md_carveout(s->mixed, stage_bytes(s), small ? 1 : per_sm, &s->carveout));
   if (s->grid > s->cta_sm_cap) {
     dfree(s, s->d_cta_sm);
     s->d_cta_sm = nullptr;
@@ -1067,7 +1074,8 @@ cudaError_t launch_persistent(md_system* s, const KParams& p) {
     kp.sharedMemBytes = (unsigned)smem;
     kp.kernelParams = args;
     cudaError_t e = cudaSuccess;
-    if (!s->gexec || s->g_grid != s->grid || s->g_block != block || s->g_smem != smem) {
+    if (!s->gexec || s->g_grid != s->grid || s->g_block != block || s->g_smem != smem ||
+        s->g_carveout != s->carveout) {
       drop_graph(s);
       e = cudaFuncSetAttribute(kp.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e == cudaSuccess) e = cudaGraphCreate(&s->graph, 0);
@@ -1076,12 +1084,18 @@ cudaError_t launch_persistent(md_system* s, const KParams& p) {
         cudaKernelNodeAttrValue v = {};
         v.cooperative = 1;
         e = cudaGraphKernelNodeSetAttribute(s->gnode, cudaKernelNodeAttributeCooperative, &v);
+        if (e == cudaSuccess) {
+          cudaKernelNodeAttrValue c = {};
+          c.sharedMemCarveout = (unsigned)s->carveout;
+          e = cudaGraphKernelNodeSetAttribute(s->gnode, cudaKernelNodeAttributePreferredSharedMemoryCarveout, &c);
+        }
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&s->gexec, s->graph, 0);
       if (e == cudaSuccess) {
         s->g_grid = s->grid;
         s->g_block = block;
         s->g_smem = smem;
+        s->g_carveout = s->carveout;
       }
     } else {
       e = cudaGraphExecKernelNodeSetParams(s->gexec, s->gnode, &kp);
@@ -1096,7 +1110,7 @@ cudaError_t launch_persistent(md_system* s, const KParams& p) {
     drop_graph(s);
     s->use_graph = false;
   }
-  return md_launch_persistent(s->mixed, p, s->grid, block, smem, s->stream);
+  return md_launch_persistent(s->mixed, p, s->grid, block, smem, s->carveout, s->stream);
 }
 
 // Run the persistent kernel for one operation, growing the neighbour list

@@ -218,9 +218,12 @@ struct KParams {
 };
 
 // Host-side launchers (md_kernel.cu).
-cudaError_t md_launch_persistent(bool mixed, const KParams& p, int grid, int block, size_t smem, cudaStream_t s);
+cudaError_t md_launch_persistent(bool mixed, const KParams& p, int grid, int block, size_t smem, int carveout,
+                                 cudaStream_t s);
 cudaError_t md_launch_log_records(bool mixed, const KParams& p, int nslots, int block, cudaStream_t s);
 cudaError_t md_occupancy(bool mixed, int block, size_t smem, int* blocks_per_sm);
+// the share of an SM's shared memory (percent) that blocks_per_sm CTAs of the persistent kernel take
+cudaError_t md_carveout(bool mixed, size_t smem, int blocks_per_sm, int* percent);
 const void* md_persistent_fn(bool mixed);
 cudaError_t md_launch_barrier_selftest(const KParams& p, int blocks, cudaStream_t s);
 // Message returned by md_last_error(NULL) on this host thread (md_api.cu).

@@ -2009,12 +2009,29 @@ cudaError_t md_launch_barrier_selftest(const KParams& p, int blocks, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t md_launch_persistent(bool mixed, const KParams& p, int grid, int block, size_t smem, cudaStream_t s) {
+cudaError_t md_launch_persistent(bool mixed, const KParams& p, int grid, int block, size_t smem, int carveout,
+                                 cudaStream_t s) {
   void* args[] = {(void*)&p};
   const void* fn = mixed ? (const void*)kamd::md_persistent<true> : (const void*)kamd::md_persistent<false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, smem, s);
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[1].val.sharedMemCarveout = (unsigned)carveout;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  e = cudaLaunchKernelExC(&cfg, fn, args);
+  if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+  cudaGetLastError();  // the split leaves no room for the grid: let the driver choose it
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 const void* md_persistent_fn(bool mixed) {
@@ -2026,4 +2043,18 @@ cudaError_t md_occupancy(bool mixed, int block, size_t smem, int* blocks_per_sm)
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, block, smem);
+}
+
+cudaError_t md_carveout(bool mixed, size_t smem, int blocks_per_sm, int* percent) {
+  cudaFuncAttributes fa;
+  int dev = 0, per_sm = 0, reserved = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, md_persistent_fn(mixed));
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t need = (int64_t)blocks_per_sm * (int64_t)(smem + fa.sharedSizeBytes + (size_t)reserved);
+  *percent = (int)((100 * need + per_sm - 1) / per_sm);
+  if (*percent > 100) *percent = 100;
+  return cudaSuccess;
 }
