@@ -52,7 +52,7 @@ typedef enum {
 typedef enum {
     MD_PREC_FP64 = 0,  /* positions, velocities, forces and pair arithmetic in FP64 */
     MD_PREC_MIXED = 1  /* 64-bit fixed-point positions, FP32 velocities, forces and pair
-                          arithmetic, FP64 energy/virial/momentum reductions */
+                          arithmetic, FP64 energy/virial reductions */
 } md_precision;
 
 typedef enum {
@@ -74,7 +74,8 @@ typedef struct {
 /* Tuning knobs (chosen by md_autotune or set by hand). Changing them never
  * changes the physics except through the order of floating-point sums. */
 typedef struct {
-    int threads_per_atom; /* 1, 2, 4 or 8 lanes share one particle's neighbour loop */
+    int threads_per_atom; /* 1, 2, 4 or 8 lanes share one particle's neighbour loop (FP64: at
+                             least four do, whatever is asked for) */
     int block_size;       /* 128, 256 or 512 threads per CTA of the persistent kernel */
     double skin;          /* inner list: radius r_c,ab + skin, pruned from the outer list
                              once any particle moved skin/2 since the last prune */
