@@ -1343,7 +1343,11 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
     __syncthreads();
     const int ncand = s_ub[nu];
     const int npart = s_pb[nrows];
-    if (npart == 0) continue;  // empty group: no particle needs a list
+    if (npart == 0) {  // empty group: no particle needs a list
+      // (the next group, maybe of a replica with more rows or cells, overwrites what a slower warp has yet to read above)
+      __syncthreads();
+      continue;
+    }
     if (ncand > stage_cap) {
       // more candidates than the staging area holds: flag and skip (the host regrows it)
       if (threadIdx.x == 0) raise_flag(p, MD_FLAG_OVERFLOW);

@@ -116,3 +116,29 @@ def test_one_replica_under_nose_hoover_equals_a_batch_member(prec, kind, n, tpa)
         last = lb if len(lb) == len(la) else lb[3::4]
         assert all(np.array_equal(la[f], last[f]) for f in la.dtype.names if f != "step")
     assert np.all(np.isfinite(la["T"])) and np.all(la["T"] > 0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_planar_batch_of_unequal_groups_equals_its_members(prec):
+    """Replicas in a plane at three densities: their list-build groups have unequal numbers of rows, and the
+    groups off the plane are empty, so a CTA passes from an empty group to one of another shape. Each replica
+    is bitwise its stand-alone run."""
+    ns = [[400, 90, 900, 60, 250][k % 5] for k in range(40)]
+    rho = [[1.2, 0.1, 0.6][k % 3] for k in range(40)]
+    Ts = [[0.1, 1.5, 0.4, 0.8][k % 4] for k in range(40)]
+    Ls = [float(np.sqrt(n / d)) for n, d in zip(ns, rho)]
+    types = [wl.ka_types(n, 7 + k).astype(np.int32) for k, n in enumerate(ns)]
+
+    def run(n, L, t, T):
+        with kamd.System(n, L, t, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec, ndim=2) as s:
+            s.set_tuning(threads_per_atom=8, block_size=256, skin=0.3, skin_outer=0.3)
+            s.init_lattice(T, seed=13)
+            s.step_nve(0.004, 60)
+            return s.get_state()
+
+    p, v, img = run(ns, Ls, np.concatenate(types), Ts)
+    off = np.concatenate([[0], np.cumsum(ns)])
+    for k in (0, 1, 2, 3, 4, 5, 17, 38, 39):
+        q, w, j = run(ns[k], Ls[k], types[k], Ts[k])
+        at = slice(off[k], off[k + 1])
+        assert np.array_equal(q, p[at]) and np.array_equal(w, v[at]) and np.array_equal(j, img[at]), k
