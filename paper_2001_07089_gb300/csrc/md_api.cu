@@ -382,6 +382,10 @@ __global__ void __launch_bounds__(MSD_THREADS) k_msd_final(int nblocks, int ntyp
 #define RDF_CELLS 4
 #define RDF_PART 16  // particles of a unit that are tested in one go
 #define RDF_WARPS 8
+// pairs that a warp bins before it moves the CTA's 32-bit counts to the 64-bit
+// histogram: a count stays below 2 RDF_WARPS (RDF_FLUSH + 32), a million, however
+// large the system (a warp takes about 16 000 pairs in all at N = 10^6 and 4 sigma)
+#define RDF_FLUSH 65536
 struct RdfArgs {
   bool mixed;
   int64_t ntot;
@@ -400,6 +404,17 @@ struct RdfWarp {
   int j[64];
   int c[64];
 };
+
+// The CTA's counts so far, moved by one warp: the exchange leaves the other
+// warps free to go on counting.
+__device__ __noinline__ void rdf_flush(unsigned int* sh_h, int n, unsigned long long* h) {
+  __syncwarp();
+  for (int t = threadIdx.x & 31; t < n; t += 32) {
+    const unsigned int v = atomicExch(&sh_h[t], 0u);
+    if (v) atomicAdd(&h[t], (unsigned long long)v);
+  }
+  __syncwarp();
+}
 
 template <bool REL>
 __device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfWarp& W, unsigned int* sh_h, bool priv, int r,
@@ -484,7 +499,13 @@ __device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfW
         W.c[e] = k | ((ti == tj ? ti : 2) << 8);
       }
       count += __popc(m);
-      if (count >= 32) bin(32);
+      if (count >= 32) {
+        bin(32);
+        if (head >= RDF_FLUSH) {
+          if (priv) rdf_flush(sh_h, 3 * a.nbins, a.hist + (int64_t)r * 3 * a.nbins);
+          head &= 63;
+        }
+      }
     }
   }
 }
@@ -513,6 +534,7 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   const float edge = (float)(err / a.dr + 1e-6 * a.nbins), invdr = (float)(1.0 / a.dr);
   const float rmax2f = (float)((rmax + 2.0 * err) * (rmax + 2.0 * err) * (1.0 + 1e-6));
   RdfWarp& W = sh_w[warp];
+  int head = 0, count = 0;  // the queue; head also counts the pairs binned since the last flush
   for (int u = b * RDF_WARPS + warp; u < units; u += a.blocks_per_rep * RDF_WARPS) {
     int s0, s1, x0 = 0, cy = 0, cz = 0, g = 0;
     if (all) {
@@ -539,7 +561,6 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
                           : make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), t);
       }
       __syncwarp();
-      int head = 0, count = 0;
       auto scan = [&](int lo, int n, bool own) {
         if (rel) rdf_scan<true>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
         else rdf_scan<false>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
