@@ -96,6 +96,7 @@ struct md_system {
   int64_t rdf_nbins = 0;
   double rdf_dr = 0.0;
   int64_t rdf_meas = 0;
+  std::vector<int32_t> rdf_blk;  // first CTA of each replica (see md_rdf)
   double* d_msd_part = nullptr;
   unsigned long long* d_count = nullptr;
   size_t bytes = 0;  // device bytes currently held (dalloc/dfree)
@@ -368,30 +369,47 @@ __global__ void __launch_bounds__(MSD_THREADS) k_msd_final(int nblocks, int ntyp
 // one row, and the half of the rows around theirs that makes each pair of rows
 // meet once (of its own row, the slots after each particle's). Row members are
 // read 32 at a time, one per lane, straight from the gather copy, and tested in
-// FP32 against each particle of the unit; pairs within rmax (about one in ten)
+// FP32 against each particle of the unit; pairs within rmax (one in six to nine)
 // wait in a queue until a full warp of them is binned. The bin follows from the
 // FP32 distance unless that lies within its own error of a bin edge; such pairs
-// (about one in a thousand at dr = 0.01) are binned from the exact positions in
+// (about three in a thousand at dr = 0.01) are binned from the exact positions in
 // FP64. So the counts are those of the exact distances, and GB300's slow FP64
 // unit, which computed every pair's difference, root and quotient before, has
 // next to nothing to do. Cells are those of the last list build; every particle
 // has moved less than half the outer skin since, so rows are reached out to
 // rmax + skin. A replica with too few cells for that is one row of all its slots.
-// Measured at N = 10^6, 400 bins to 4 sigma, with the MSD call: 30.6 ms -> 3.5 ms.
+// k_rdf_units lists the units that hold particles: most cells of a dilute box or
+// of a plane hold none, and walking them took 1.3 s for 1000 particles in a box
+// of 1024 cells per edge, where the whole call now takes 87 us.
+// 400 bins to 4 sigma at N = 10^6: 2.6 ms (27 ms in FP64 throughout). What bounds
+// a large system is the tests' issue slots, one below 10^5 particles the chain of
+// one unit; units of 4 cells were slower at every N: 20 000 particles 424 us
+// (now 254), 10^6 2836 us (units of 1 cell 3232).
 #define RDF_SMEM_BINS 1024
-#define RDF_CELLS 4
+#define RDF_CELLS 2
 #define RDF_PART 16  // particles of a unit that are tested in one go
 #define RDF_WARPS 8
 // pairs that a warp bins before it moves the CTA's 32-bit counts to the 64-bit
-// histogram: a count stays below 2 RDF_WARPS (RDF_FLUSH + 32), a million, however
-// large the system (a warp takes about 16 000 pairs in all at N = 10^6 and 4 sigma)
+// histogram (at N = 10^6 and 4 sigma it bins about 16 000 in all), and candidates
+// between two looks at that number: a count stays below 2 RDF_WARPS (RDF_FLUSH +
+// RDF_PART RDF_LOOK), 2.7e8, however large the system
 #define RDF_FLUSH 65536
+#define RDF_LOOK 1048576
+// slots at whose multiples units are cut, so that no warp takes much more than
+// this many particles, however many a cell holds (a droplet in a box of 1024
+// wide cells per edge)
+#define RDF_CUT 256
 struct RdfArgs {
   bool mixed;
   int64_t ntot;
-  int nbins, blocks_per_rep;
+  int nbins, ndim, nrep;
   double dr, skin;
   const RepDev* reps;
+  const int32_t* tile_rep;
+  const uint4* xbq;   // positions at the last list build: the cells that slots are sorted by
+  int32_t* unit;      // first slots of the units, replica r's from unit[off]
+  int32_t* nunits;    // per replica
+  const int32_t* blk; // first CTA of each replica, and the number of CTAs (one replica: not read)
   const uint4* pq;
   const uint64_t* pfx;
   const double4_32a* p4;
@@ -407,7 +425,7 @@ struct RdfWarp {
 
 // The CTA's counts so far, moved by one warp: the exchange leaves the other
 // warps free to go on counting.
-__device__ __noinline__ void rdf_flush(unsigned int* sh_h, int n, unsigned long long* h) {
+__device__ __forceinline__ void rdf_flush(unsigned int* sh_h, int n, unsigned long long* h) {
   __syncwarp();
   for (int t = threadIdx.x & 31; t < n; t += 32) {
     const unsigned int v = atomicExch(&sh_h[t], 0u);
@@ -475,6 +493,7 @@ __device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfW
       y = (float)(int)(q.y - ref.y) * sc;
       z = (float)(int)(q.z - ref.z) * sc;
     }
+#pragma unroll 4
     for (int k = 0; k < np; ++k) {
       const float4 P = W.pos[k];
       float dx, dy, dz;
@@ -499,22 +518,80 @@ __device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfW
         W.c[e] = k | ((ti == tj ? ti : 2) << 8);
       }
       count += __popc(m);
-      if (count >= 32) {
-        bin(32);
-        if (head >= RDF_FLUSH) {
-          if (priv) rdf_flush(sh_h, 3 * a.nbins, a.hist + (int64_t)r * 3 * a.nbins);
-          head &= 63;
-        }
-      }
+      if (count >= 32) bin(32);
     }
   }
+}
+
+// Layers of cells that hold the partners within rmax; false: too few cells for
+// that, every slot of the replica is a candidate.
+__device__ __host__ __forceinline__ bool rdf_layers(double rmax, double skin, int nc, float cellw, int* layers) {
+  *layers = nc > 0 ? (int)ceil((rmax + skin) * (1.0 + 1e-6) / (double)cellw) : 0;
+  return nc > 0 && 2 * *layers + 1 <= nc;
+}
+
+// Cell of a slot at the last list build (the binning that sorted the slots).
+__device__ __forceinline__ int3 rdf_cell(const uint4& x, int nc) {
+  return make_int3((int)(((uint64_t)x.x * (uint64_t)nc) >> 32), (int)(((uint64_t)x.y * (uint64_t)nc) >> 32),
+                   (int)(((uint64_t)x.z * (uint64_t)nc) >> 32));
+}
+
+// First slots of the units. A warp is a tile; the CTA's units of a replica are
+// listed together and in order, so that the warps of a CTA of k_rdf work side by
+// side and share rows in L1 (the order of the CTAs is left open: counts do not
+// depend on it).
+#define RDF_LIST 1024
+__global__ void __launch_bounds__(RDF_LIST) k_rdf_units(RdfArgs a) {
+  __shared__ int sh_r[RDF_LIST / 32], sh_n[RDF_LIST / 32], sh_base[RDF_LIST / 32];
+  const int64_t i = (int64_t)blockIdx.x * RDF_LIST + threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool in = i < a.ntot;
+  const int r = in ? a.tile_rep[i >> 5] : -1;
+  const RepDev& R = a.reps[in ? r : 0];
+  const int64_t k = i - R.off;
+  bool first = false;
+  int layers;
+  if (in && k < R.n) {
+    if (!rdf_layers(a.dr * a.nbins, a.skin, R.nc, R.cellw, &layers)) {
+      first = k % RDF_PART == 0;
+    } else if (k == 0 || i % RDF_CUT == 0) {
+      first = true;
+    } else {
+      const int3 c = rdf_cell(a.xbq[i], R.nc), d = rdf_cell(a.xbq[i - 1], R.nc);
+      first = c.x / RDF_CELLS != d.x / RDF_CELLS || c.y != d.y || c.z != d.z;
+    }
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, first);
+  if (lane == 0) {
+    sh_r[warp] = r;
+    sh_n[warp] = __popc(m);
+  }
+  __syncthreads();
+  // the tiles of this one's replica: units in those before it, and in all
+  const bool same = sh_r[lane] == r;
+  const unsigned tiles = __ballot_sync(0xffffffffu, same);
+  const int before = __reduce_add_sync(0xffffffffu, same && lane < warp ? sh_n[lane] : 0);
+  const int all = __reduce_add_sync(0xffffffffu, same ? sh_n[lane] : 0);
+  const int head = __ffs(tiles) - 1;
+  if (warp == head && lane == 0 && in) sh_base[warp] = atomicAdd(&a.nunits[r], all);
+  __syncthreads();
+  if (first) a.unit[R.off + sh_base[head] + before + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
 }
 
 __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   __shared__ unsigned int sh_h[3 * RDF_SMEM_BINS];
   __shared__ RdfWarp sh_w[RDF_WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = blockIdx.x / a.blocks_per_rep, b = blockIdx.x - r * a.blocks_per_rep;
+  int r = 0, b = blockIdx.x, nblk = gridDim.x;
+  if (a.nrep > 1) {
+    int hi = a.nrep;  // blk[r] <= blockIdx.x < blk[hi]
+    while (hi - r > 1) {
+      const int mid = (r + hi) >> 1;
+      if (a.blk[mid] <= b) r = mid; else hi = mid;
+    }
+    nblk = a.blk[r + 1] - a.blk[r];
+    b -= a.blk[r];
+  }
   const RepDev& R = a.reps[r];
   const bool priv = a.nbins <= RDF_SMEM_BINS;
   if (priv)
@@ -522,10 +599,9 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   __syncthreads();
   const double rmax = a.dr * a.nbins;
   const int nc = R.nc;
-  const int layers = nc > 0 ? (int)ceil((rmax + a.skin) * (1.0 + 1e-6) / (double)R.cellw) : 0;
-  const bool all = nc == 0 || 2 * layers + 1 > nc;
-  const int runs = all ? 0 : (nc + RDF_CELLS - 1) / RDF_CELLS;  // units per row of cells
-  const int units = all ? (R.n + RDF_PART - 1) / RDF_PART : runs * nc * nc;
+  int layers;
+  const bool all = !rdf_layers(rmax, a.skin, nc, R.cellw, &layers);
+  const int units = a.nunits[r];
   const bool rel = !all && 2 * (RDF_CELLS + layers + 1) < nc;
   // the FP32 distance is off by less than err: the rounding of coordinates of
   // at most `span`, and the words' own error
@@ -535,19 +611,18 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   const float rmax2f = (float)((rmax + 2.0 * err) * (rmax + 2.0 * err) * (1.0 + 1e-6));
   RdfWarp& W = sh_w[warp];
   int head = 0, count = 0;  // the queue; head also counts the pairs binned since the last flush
-  for (int u = b * RDF_WARPS + warp; u < units; u += a.blocks_per_rep * RDF_WARPS) {
-    int s0, s1, x0 = 0, cy = 0, cz = 0, g = 0;
+  for (int64_t u = b * RDF_WARPS + warp; u < units; u += (int64_t)nblk * RDF_WARPS) {
+    const int s0 = a.unit[R.off + u];
+    int s1, x0 = 0, cy = 0, cz = 0, g = 0;
     if (all) {
-      s0 = (int)R.off + u * RDF_PART;
       s1 = min(s0 + RDF_PART, (int)R.off + R.n);
     } else {
-      x0 = (u % runs) * RDF_CELLS;
-      cy = (u / runs) % nc;
-      cz = u / (runs * nc);
+      const int3 c = rdf_cell(a.xbq[s0], nc);
+      x0 = c.x / RDF_CELLS * RDF_CELLS;
+      cy = c.y;
+      cz = c.z;
       g = min(RDF_CELLS, nc - x0);
-      const int32_t* cs = a.cstart + R.cs0 + (cz * nc + cy) * nc + x0;
-      s0 = cs[0];
-      s1 = cs[g];
+      s1 = min(a.cstart[R.cs0 + (cz * nc + cy) * nc + x0 + g], s0 / RDF_CUT * RDF_CUT + RDF_CUT);
     }
     for (int i0 = s0; i0 < s1; i0 += RDF_PART) {
       const int np = min(RDF_PART, s1 - i0);
@@ -562,8 +637,17 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
       }
       __syncwarp();
       auto scan = [&](int lo, int n, bool own) {
-        if (rel) rdf_scan<true>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
-        else rdf_scan<false>(a, R, W, sh_h, priv, r, i0, np, ref, lo, n, own, rmax2f, invdr, edge, head, count);
+        do {
+          const int m = min(n, RDF_LOOK);
+          if (rel) rdf_scan<true>(a, R, W, sh_h, priv, r, i0, np, ref, lo, m, own, rmax2f, invdr, edge, head, count);
+          else rdf_scan<false>(a, R, W, sh_h, priv, r, i0, np, ref, lo, m, own, rmax2f, invdr, edge, head, count);
+          if (head >= RDF_FLUSH) {
+            if (priv) rdf_flush(sh_h, 3 * a.nbins, a.hist + (int64_t)r * 3 * a.nbins);
+            head &= 63;
+          }
+          lo += m;
+          n -= m;
+        } while (n > 0);
       };
       if (all) {
         scan(i0, (int)R.off + R.n - i0, true);
@@ -571,15 +655,32 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
         const int len = min(2 * layers + g, nc);
         const int a0 = len == nc ? 0 : (x0 - layers + nc) % nc;
         const int over = max(a0 + len - nc, 0);
-        for (int oz = 0; oz <= layers; ++oz)
-          for (int oy = oz == 0 ? 0 : -layers; oy <= layers; ++oy) {
+        // rows (oy, oz): (0..layers, 0), then (-layers..layers, 1..layers); their
+        // runs [a0, a0 + len) of cells, in two parts where they pass the box
+        // edge, are looked up by one lane each
+        const int wide = 2 * layers + 1;
+        const int rows = layers + 1 + (a.ndim == 3 ? layers * wide : 0);
+        for (int q0 = 0; q0 < rows; q0 += 32) {
+          const int q = q0 + lane;
+          int lo0 = 0, n0 = 0, lo1 = 0, n1 = 0;
+          if (q < rows) {
+            const int oz = q <= layers ? 0 : 1 + (q - layers - 1) / wide;
+            const int oy = q <= layers ? q : (q - layers - 1) % wide - layers;
             const int32_t* cs = a.cstart + R.cs0 + (((cz + oz) % nc) * nc + (cy + oy + nc) % nc) * nc;
-            // the run [a0, a0 + len) of cells, in two parts where it passes the box edge
-            for (int part = 0; part < (over > 0 ? 2 : 1); ++part) {
-              const int lo = cs[part ? 0 : a0], n = cs[part ? over : a0 + len - over] - lo;
-              if (n > 0) scan(lo, n, oz == 0 && oy == 0);
+            lo0 = cs[a0];
+            n0 = cs[a0 + len - over] - lo0;
+            if (over > 0) {
+              lo1 = cs[0];
+              n1 = cs[over] - lo1;
             }
           }
+          for (int part = 0; part < 2; ++part)
+            for (unsigned m = __ballot_sync(0xffffffffu, (part ? n1 : n0) > 0); m; m &= m - 1u) {
+              const int from = __ffs(m) - 1;
+              scan(__shfl_sync(0xffffffffu, part ? lo1 : lo0, from), __shfl_sync(0xffffffffu, part ? n1 : n0, from),
+                   q0 + from == 0);
+            }
+        }
       }
       scan(-1, 0, false);
     }
@@ -1650,21 +1751,50 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
   a.mixed = s->mixed;
   a.ntot = s->ntot;
   a.nbins = (int)nbins;
+  a.ndim = s->ndim;
+  a.nrep = s->nrep;
   a.dr = dr;
   a.skin = s->tun.skin_outer;
   a.reps = s->d_reps;
+  a.tile_rep = s->d_tile_rep;
+  a.xbq = s->d_xbq;
+  // (two arrays of a rebuild, which has no use for them now: 32 entries per replica at least)
+  a.unit = s->d_scat;
+  a.nunits = s->d_cellof;
+  a.blk = s->d_cellof + s->nrep;
   a.pq = s->d_pq[s->ctl.cur];
   a.pfx = s->d_pfx;
   a.p4 = s->d_p4[s->ctl.cur];
   a.cstart = s->d_cstart;
   a.hist = s->d_rdf;
-  // about eight CTAs per SM over all replicas, at most one warp per unit
-  // (a unit holds 8 particles or more in anything but a gas)
-  int64_t nmax = 0;
-  for (int64_t n : s->n_per) nmax = std::max(nmax, n);
-  a.blocks_per_rep = (int)std::max<int64_t>(
-      1, std::min<int64_t>((nmax / 8 + RDF_WARPS) / RDF_WARPS, (8 * (int64_t)s->nsm + s->nrep - 1) / s->nrep));
-  k_rdf<<<(unsigned)(a.blocks_per_rep * (int64_t)s->nrep), 32 * RDF_WARPS, 0, s->stream>>>(a);
+  // about eight CTAs per SM, shared out over the replicas by their candidate
+  // pairs, at most one warp per unit (a unit holds 8 particles or more in
+  // anything but a gas). With as many for each replica, one of 120 000 particles
+  // among 1215 of two had one CTA: all pairs to L/2 6.4 s, now 27 ms.
+  std::vector<double> work((size_t)s->nrep);
+  double total = 0.0;
+  for (int r = 0; r < s->nrep; ++r) {
+    const RepDev& R = s->reps[r];
+    int l;
+    double share = 0.5;
+    if (rdf_layers(dr * nbins, a.skin, R.nc, R.cellw, &l))
+      share = std::min(0.5, (2.0 * l + RDF_CELLS) * (l + 1.0) * (s->ndim == 3 ? 2.0 * l + 1.0 : 1.0) /
+                                std::pow((double)R.nc, (double)s->ndim));
+    work[r] = (double)R.n * (double)R.n * share;
+    total += work[r];
+  }
+  s->rdf_blk.assign(1, 0);
+  for (int r = 0; r < s->nrep; ++r) {
+    const int64_t most = (s->n_per[r] / 8 + RDF_WARPS) / RDF_WARPS;
+    const int64_t fair = (int64_t)std::ceil(8.0 * s->nsm * work[r] / total);
+    s->rdf_blk.push_back(s->rdf_blk.back() + (int32_t)std::max<int64_t>(1, std::min(most, fair)));
+  }
+  CK(cudaMemsetAsync(a.nunits, 0, 4 * (size_t)s->nrep, s->stream));
+  if (s->nrep > 1)
+    CK(cudaMemcpyAsync(s->d_cellof + s->nrep, s->rdf_blk.data(), 4 * s->rdf_blk.size(), cudaMemcpyHostToDevice, s->stream));
+  k_rdf_units<<<blocks_for(s->ntot, RDF_LIST), RDF_LIST, 0, s->stream>>>(a);
+  CK(cudaGetLastError());
+  k_rdf<<<(unsigned)s->rdf_blk.back(), 32 * RDF_WARPS, 0, s->stream>>>(a);
   CK(cudaGetLastError());
   s->rdf_meas += 1;
   if (g) {

@@ -72,3 +72,79 @@ def test_long_rows_count_as_the_oracle(prec):
         p, _, _ = s.get_state()
     ref = counts(oracle.rdf(p, types, L, dr, nbins), types, L, dr, nbins)
     assert np.array_equal(counts(g, types, L, dr, nbins), ref)
+
+
+def seconds(s, dr, nbins):
+    import time
+    best = np.inf
+    for _ in range(4):
+        t = time.perf_counter()
+        s.rdf(dr, nbins, reset=True)
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+def test_cost_follows_the_particles_not_the_cells():
+    """10 000 particles in a box of 620 cells per edge cost what they do in one of 62: the pairs are far fewer,
+    and walking the empty cells alone took 200 times as long."""
+    n = 10000
+    types = wl.ka_types(n, 6).astype(np.int32)
+    t = []
+    for L in (100.0, 1000.0):
+        with system(n, L, types, "mixed") as s:
+            s.set_state(wl.uniform_positions(n, L, 6))
+            t.append(seconds(s, 0.01, 400))
+    assert t[1] < 10 * t[0], t
+
+
+def test_largest_replica_of_a_batch_gets_its_share_of_the_gpu():
+    """120 000 particles and all pairs to L/2 cost about as much with 255 pairs of particles beside them as alone."""
+    n, small = 120000, 255
+    L = wl.box_length(n)
+    types = wl.ka_types(n, 3).astype(np.int32)
+    pos = np.concatenate([wl.uniform_positions(n, L, 3), wl.uniform_positions(2 * small, L, 4)])
+    t, g = [], []
+    for k in (0, small):
+        m = n + 2 * k
+        with system([n] + [2] * k if k else n, [L] * (k + 1) if k else L,
+                    np.concatenate([types, np.tile(np.int32([0, 1]), k)]), "mixed") as s:
+            s.set_state(pos[:m])
+            t.append(seconds(s, 0.0499 * L, 10))
+            g.append(s.rdf(0.0499 * L, 10, reset=True)[:2] * (k + 1))  # like pairs: the large replica's
+    assert np.allclose(g[0], g[1], rtol=1e-12)
+    assert t[1] < 10 * t[0], t
+
+
+@pytest.mark.parametrize("ndim,L", [(3, 30.0), (3, 60.0), (2, 150.0)])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_dilute_boxes_and_droplets(prec, ndim, L):
+    """Half the particles anywhere in the box, half in a dense droplet on its corner: empty cells, cells with
+    one particle, and runs of cells long enough to be cut, after steps that move particles from their cells."""
+    n, m = 3000, {3: 14, 2: 50}[ndim]
+    half = 0.5 * (n / 2) ** (1 / ndim)  # half the droplet's edge at number density 1
+    k = int(np.ceil((n // 2) ** (1 / ndim)))
+    site = np.stack(np.unravel_index(np.arange(n // 2), (k,) * ndim), 1)
+    drop = (site + 0.5) * (2 * half / k) - half
+    gas = (np.stack(np.unravel_index(np.arange(m ** ndim), (m,) * ndim), 1) + 0.5) * (L / m) - 0.5 * L
+    gas = gas[np.any(np.abs(gas) > half + 1.5, axis=1)]
+    gas = gas[np.random.default_rng(8).permutation(len(gas))[:n - n // 2]]
+    gas += np.random.default_rng(9).uniform(-0.5, 0.5, gas.shape)
+    pos = np.full((n, 3), 0.5 * L)
+    pos[:, :ndim] = np.concatenate([drop, gas]) % L
+    types = wl.ka_types(n, 8).astype(np.int32)
+    dr, nbins = 0.02, 200
+    with system(n, L, types, prec, ndim=ndim) as s:
+        s.set_state(pos)
+        s.step_nvt(0.002, 1, 0.5, kind=kamd.MD_NVT_RESAMPLE, param=1, seed=3)
+        s.step_nve(0.002, 20)
+        g = s.rdf(dr, nbins, reset=True)
+        p, _, _ = s.get_state()
+    ref = oracle.rdf(p, types, L, dr, nbins, ndim=ndim)
+    k = np.arange(nbins)
+    na = int(np.sum(types == 0))
+    nb = n - na
+    shell = 4 / 3 * np.pi * ((k + 1.0) ** 3 - k ** 3) * dr ** 3 if ndim == 3 else np.pi * (2 * k + 1.0) * dr ** 2
+    w = np.outer([na * (na - 1.0), nb * (nb - 1.0), na * float(nb)], shell / L ** ndim)
+    c, r = np.rint(g * w), np.rint(ref * w)
+    assert r.sum() > 10 * n and np.max(np.abs(g * w - c)) < 1e-6
+    assert np.array_equal(c, r)
