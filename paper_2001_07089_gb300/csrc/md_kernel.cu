@@ -45,7 +45,7 @@ struct Shared {
   double4_32a tabd[MD_MAXTYPES * MD_MAXTYPES];
   double2 tabed[MD_MAXTYPES * MD_MAXTYPES];
   double red[16][MD_NPART];
-  int scan[32];
+  long long scan[32];
   RepDev lone;  // Nose-Hoover steps of a single replica: this CTA's copy (see reduce_phase)
   int snap;
   unsigned gen;  // grid barrier generation this CTA waits for next (thread 0)
@@ -1009,29 +1009,31 @@ __device__ __forceinline__ void cell_of_pos(const KParams& p, const RepDev& R, i
   cz = (int)(((uint64_t)q.z * (uint64_t)nc) >> 32);
 }
 
-// Block-wide exclusive scan of one int per thread.
-__device__ int block_exclusive_scan(Shared& sh, int v, int* total) {
+// Block-wide exclusive scan of one number per thread.
+template <class V>
+__device__ V block_exclusive_scan(Shared& sh, V v, V* total) {
+  V* const tot = reinterpret_cast<V*>(sh.scan);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  int x = v;
+  V x = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    const V y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) sh.scan[warp] = x;
+  if (lane == 31) tot[warp] = x;
   __syncthreads();
   if (warp == 0) {
-    int w = lane < nwarp ? sh.scan[lane] : 0;
+    V w = lane < nwarp ? tot[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      const V y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    if (lane < nwarp) sh.scan[lane] = w;
+    if (lane < nwarp) tot[lane] = w;
   }
   __syncthreads();
-  const int before = (warp > 0 ? sh.scan[warp - 1] : 0) + x - v;
-  *total = sh.scan[nwarp - 1];
+  const V before = (warp > 0 ? tot[warp - 1] : 0) + x - v;
+  *total = tot[nwarp - 1];
   __syncthreads();
   return before;
 }
@@ -1524,7 +1526,9 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
     int64_t carry = 0, gcarry = 0, ccarry = 0;
     for (int r0 = 0; r0 < p.nrep; r0 += blockDim.x) {
       const int r = r0 + (int)threadIdx.x;
-      int v = 0, g = 0, c = 0;
+      // (two replicas of 1024 cells per edge have 2^31 cells: their sums take 64 bits)
+      int v = 0;
+      long long g = 0, c = 0;
       if (r < p.nrep) {
         const RepDev& R = p.reps[r];
         if (R.doing_rebuild) {
@@ -1533,10 +1537,11 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
           c = R.nc * R.nc * R.nc;
         }
       }
-      int total, gtotal, ctotal;
+      int total;
+      long long gtotal, ctotal;
       const int pre = block_exclusive_scan(sh, v, &total);
-      const int gpre = block_exclusive_scan(sh, g, &gtotal);
-      const int cpre = block_exclusive_scan(sh, c, &ctotal);
+      const long long gpre = block_exclusive_scan(sh, g, &gtotal);
+      const long long cpre = block_exclusive_scan(sh, c, &ctotal);
       if (r < p.nrep) {
         p.reps[r].cell_base = carry + pre;
         p.reps[r].grp_base = gcarry + gpre;

@@ -142,3 +142,31 @@ def test_planar_batch_of_unequal_groups_equals_its_members(prec):
         q, w, j = run(ns[k], Ls[k], types[k], Ts[k])
         at = slice(off[k], off[k + 1])
         assert np.array_equal(q, p[at]) and np.array_equal(w, v[at]) and np.array_equal(j, img[at]), k
+
+
+def test_two_replicas_of_the_most_cells():
+    """Two boxes of 1024 cells per edge hold 2^31 cells between them, one more than 31 bits count. Each
+    replica's forces are the oracle's, and so after steps with rebuilds in between."""
+    import torch
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of device memory")
+    n, L = 60, 1700.0
+    pos, vel, types, _ = melted(250, 21, nsteps=200)
+    rng = np.random.default_rng(6)
+    # clusters of particles from a melt, each somewhere in its box
+    near = np.argsort(np.sum((pos - pos[0] - 1e-9) ** 2, axis=1))[:n]
+    ps = [(pos[near] - pos[0] + rng.uniform(0, L, 3)) % L for _ in range(2)]
+    t = types[near]
+    with kamd.System([n, n], [L, L], np.concatenate([t, t]), wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, "mixed") as s:
+        s.set_tuning(threads_per_atom=4, block_size=256, skin=0.2, skin_outer=0.2)
+        s.set_state(np.concatenate(ps), np.concatenate([vel[near], -vel[near]]))
+        f = [s.forces()[0]]
+        s.step_nve(0.002, 40)
+        f.append(s.forces()[0])
+        p, _, _ = s.get_state()
+        assert s.info()["rebuilds"] > 2
+    for q, g in zip((np.concatenate(ps), p), f):
+        for k in range(2):
+            at = slice(k * n, (k + 1) * n)
+            ref, _, _ = oracle.forces(q[at], t, oracle.Params(wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0), L)
+            assert force_errors(g[at], ref)[0] <= 1e-4
