@@ -782,11 +782,14 @@ md_status upload_reps(md_system* s) {
   return MD_OK;
 }
 md_status upload_state(md_system* s) {
+  // (many replicas go by themselves: putting 1.6 MB of them together cost more than a second copy does)
+  if (s->reps_dirty && s->nrep > LAND_REPS) CKS(upload_reps(s));
   const size_t nr = s->reps_dirty ? sizeof(RepDev) * (size_t)s->nrep : 0;
-  s->up.resize(CTL_BYTES + nr);
+  const size_t bytes = CTL_BYTES + nr;
+  if (s->up.size() < bytes) s->up.resize(bytes);
   std::memcpy(s->up.data(), &s->ctl, sizeof(CtlDev));
   if (nr) std::memcpy(s->up.data() + CTL_BYTES, s->reps.data(), nr);
-  CK(cudaMemcpyAsync(s->d_state, s->up.data(), s->up.size(), cudaMemcpyHostToDevice, s->stream));
+  CK(cudaMemcpyAsync(s->d_state, s->up.data(), bytes, cudaMemcpyHostToDevice, s->stream));
   s->reps_dirty = false;
   return MD_OK;
 }

@@ -92,6 +92,33 @@ def test_partial_rebuilds_of_more_replicas_than_threads(prec, block):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_thousands_of_replicas_equal_their_own_runs(prec):
+    """2500 replicas, some with cells and some without, cold and hot, so that any of them rebuild together:
+    each is found among the others (bitwise its stand-alone run), and their energies come back."""
+    ns = [[30, 2, 64, 9, 100, 5, 40][k % 7] for k in range(2500)]
+    Ls = [[6.0, 12.0, 8.0][k % 3] for k in range(2500)]
+    Ts = [[0.01, 4.0, 0.5, 1.0, 0.1][k % 5] for k in range(2500)]
+    types = [np.arange(n, dtype=np.int32) % 2 for n in ns]
+    tun = dict(threads_per_atom=4, block_size=256, skin=0.2, skin_outer=0.2)
+
+    def run(n, L, t, T):
+        with kamd.System(n, L, t, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, prec) as s:
+            s.set_tuning(**tun)
+            s.init_lattice(T, seed=17)
+            s.step_nve(0.003, 30)
+            f, pe, w = s.forces()
+            return s.get_state() + (f,), np.stack([pe, w]), s.info()["rebuilds"]
+
+    x, e, rebuilds = run(ns, Ls, np.concatenate(types), Ts)
+    assert 2 * 2500 < rebuilds < 2500 * 30
+    off = np.concatenate([[0], np.cumsum(ns)])
+    for k in (0, 1, 2, 3, 30, 31, 32, 78, 79, 80, 511, 1023, 1024, 1025, 2448, 2498, 2499):
+        y, d, _ = run(ns[k], Ls[k], types[k], Ts[k])
+        assert all(np.array_equal(a, b[off[k]:off[k + 1]]) for a, b in zip(y, x)), k
+        assert np.array_equal(d[:, 0], e[:, k]), k
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("kind", [kamd.MD_NVT_NOSE_HOOVER, kamd.MD_NVT_NOSE_HOOVER_EXACT], ids=["nh", "nh-exact"])
 @pytest.mark.parametrize("n,tpa", [(250, 8), (1000, 1), (32768, 4), (32800, 2)])
 def test_one_replica_under_nose_hoover_equals_a_batch_member(prec, kind, n, tpa):
