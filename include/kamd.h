@@ -343,7 +343,7 @@ md_status md_selftest_barrier(md_system* sys, double timeout_s);
  * allocator and its implicit synchronisation, and hosts that give the
  * library a fixed memory budget. Every other caller should use md_forces.
  *
- * All scratch lives in one static device array of 1.4 MiB that every GPU
+ * All scratch lives in one static device array of 1.5 MiB that every GPU
  * which loads the library holds until the process exits. Hence the limits:
  * 2 <= n <= 131072 particles and at most 32 cells per box edge (larger boxes
  * use larger cells); larger n is rejected with MD_ERR_INVALID_ARG and a
