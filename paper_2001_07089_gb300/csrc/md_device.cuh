@@ -87,7 +87,14 @@ __device__ __forceinline__ double rcp_f64(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  const double z = fma(y, fma(e, e, e), y);
+  return __double2hiint(y) == 0x7ff00000 ? y : z;  // 1/0: e is NaN
+}
+
+// x < y of a sum of squares x and a positive number y, by their bit patterns
+// (as unsigned numbers: a NaN of either sign is above every y).
+__device__ __forceinline__ bool less_f64(double x, double y) {
+  return (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(y);
 }
 
 // Minimum image of one coordinate difference (the branch rule; the comparison

@@ -256,8 +256,9 @@ __device__ __forceinline__ void drift_mix(const KParams& p, const RepDev& R, int
 }
 
 // Position update of one particle, FP64 path: wrap into [0, L). Comparisons
-// are made on the bit patterns (of non-negative doubles they order alike): an
-// FP64 compare would cost as much as an FMA of that pipe.
+// are made on the bit patterns (of non-negative doubles they order alike, and as
+// unsigned numbers those of negative ones and of NaN lie above): an FP64 compare
+// would cost as much as an FMA of that pipe.
 __device__ __forceinline__ void drift_f64(const KParams& p, const RepDev& R, int64_t i, int cur, const double v[3],
                                           const double a[3], double xi, int64_t nstep) {
   const int64_t nt = p.ntot;
@@ -275,10 +276,11 @@ __device__ __forceinline__ void drift_f64(const KParams& p, const RepDev& R, int
   double xs[3] = {x.x + d[0], x.y + d[1], x.z + d[2]};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    if (__double_as_longlong(xs[c]) >= Lb) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
-    else if (__double_as_longlong(xs[c]) < 0) {
+    if ((unsigned long long)__double_as_longlong(xs[c]) < (unsigned long long)Lb) continue;  // in [0, L)
+    if (xs[c] >= R.L) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
+    else if (xs[c] < 0.0) {
       xs[c] += R.L; p.img[c * nt + i] -= 1;
-      if (__double_as_longlong(xs[c]) >= Lb) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
+      if (xs[c] >= R.L) { xs[c] -= R.L; p.img[c * nt + i] += 1; }
     }
   }
   p.p4[cur ^ 1][i] = make_double4_32a(xs[0], xs[1], xs[2], x.w);
@@ -403,7 +405,7 @@ __device__ __forceinline__ void pair_f64(const Shared& sh, const double4_32a& pi
   const double dx = image_f64(pi.x - pj.x, L, hLb), dy = image_f64(pi.y - pj.y, L, hLb), dz = image_f64(pi.z - pj.z, L, hLb);
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
   const double4_32a c = sh.tabd[tt];
-  if (__double_as_longlong(r2) < __double_as_longlong(c.x)) {
+  if (less_f64(r2, c.x)) {
     const double y = rcp_f64(r2);
     const double y3 = y * y * y;
     const double w = y3 * fma(c.y, y3, -c.z);

@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(Scratch s, const doubl
                          dz = kamd::image_f64(zi - cand[2][h], L, hLb);
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
             const int tt = row + min((int)(word[h].w >> 30), ntypes - 1);
-            if (__double_as_longlong(r2) < __double_as_longlong(tb.rc2[tt])) {
+            if (kamd::less_f64(r2, tb.rc2[tt])) {
               const double y = kamd::rcp_f64(r2);
               const double y3 = y * y * y;
               const double w = y3 * fma(tb.c12[tt], y3, -tb.c6[tt]);

@@ -1,0 +1,77 @@
+"""The FP64 force paths (md_forces of an FP64 system and md_forces_noalloc) on inputs that their FP32 tests and
+bit-pattern comparisons have to carry: positions that are not numbers, particles in one place."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2001_07089_gb300 import kamd
+from paper_2001_07089_gb300 import workloads as wl
+from tests.helpers import force_errors, ka_params, melted
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kamd.load()
+
+
+def noalloc(pos, types, L, eps=wl.KA_EPS, sig=wl.KA_SIG, rc=wl.KA_RC):
+    import torch
+    n = len(pos)
+    f = torch.empty((n, 3), dtype=torch.float64, device="cuda")
+    e = torch.empty(2, dtype=torch.float64, device="cuda")
+    dpos = torch.tensor(pos, dtype=torch.float64, device="cuda")
+    dtyp = torch.tensor(np.asarray(types, dtype=np.uint8), device="cuda")
+    torch.cuda.synchronize()
+    kamd.md_forces_noalloc(n, dpos, dtyp, len(eps), L, eps, sig, rc, f, e[:1], e[1:],
+                           torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    return f.cpu().numpy(), float(e[0]), float(e[1])
+
+
+@pytest.mark.parametrize("bad", [np.nan, -np.nan, np.inf, -np.inf], ids=["nan", "-nan", "inf", "-inf"])
+def test_a_particle_without_a_position_acts_on_none(bad):
+    """It takes part in no pair: its force is zero, the others' and the energy are those without it, also
+    after steps, and it crosses no box edge."""
+    pos, vel, types, L = melted(1000, 22, nsteps=200)
+    pos, rest = pos.copy(), np.arange(1000) != 7
+    pos[7, 0] = bad
+    f_ref, pe_ref, _ = oracle.forces(pos[rest], types[rest], ka_params(), L)
+    f, pe, _ = noalloc(pos, types, L)
+    assert np.all(f[7] == 0.0) and force_errors(f[rest], f_ref)[0] <= 1e-12
+    assert abs(pe - pe_ref) <= 1e-12 * abs(pe_ref)
+    with kamd.System(1000, L, types, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, "fp64") as s:
+        s.set_state(pos, vel)
+        f, pe, _ = s.forces()
+        assert np.all(f[7] == 0.0) and force_errors(f[rest], f_ref)[0] <= 1e-12
+        assert abs(pe[0] - pe_ref) <= 1e-12 * abs(pe_ref)
+        s.step_nve(0.002, 10)
+        p, _, img = s.get_state()
+        f, _, _ = s.forces()
+    assert img[7, 0] == 0 and np.isnan(p[7, 0])
+    f_ref, _, _ = oracle.forces(p[rest], types[rest], ka_params(), L)
+    assert np.all(f[7] == 0.0) and force_errors(f[rest], f_ref)[0] <= 1e-12
+
+
+def test_particles_in_one_place():
+    """Two particles at the same point: infinite energy, forces that are not numbers on these two alone."""
+    pos, _, types, L = melted(1000, 22, nsteps=200)
+    pos = pos.copy()
+    pos[9] = pos[400]
+    two = np.isin(np.arange(1000), (9, 400))
+    f_ref, _, _ = oracle.forces(pos[~two], types[~two], ka_params(), L)
+    one, _, _ = oracle.forces(pos[np.arange(1000) != 9], types[np.arange(1000) != 9], ka_params(), L)
+    other, _, _ = oracle.forces(pos[np.arange(1000) != 400], types[np.arange(1000) != 400], ka_params(), L)
+    # every other particle feels both
+    f_ref = np.delete(one, 399, axis=0) + np.delete(other, 9, axis=0) - f_ref
+    with kamd.System(1000, L, types, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, "fp64") as s:
+        s.set_state(pos)
+        f, pe, w = s.forces()
+        results = [(f, pe[0], w[0]), noalloc(pos, types, L)]
+    for f, pe, w in results:
+        assert pe == np.inf and w == np.inf
+        assert np.all(np.isnan(f[two])) and force_errors(f[~two], f_ref)[0] <= 1e-11
