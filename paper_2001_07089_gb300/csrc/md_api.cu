@@ -25,6 +25,7 @@ struct md_system {
   std::vector<int64_t> n_type0;  // particles of type 0 per replica
   double eps[16] = {0}, sig[16] = {0}, rc[16] = {0};
   double mass = 1.0;
+  double unit = 1.0;  // FP64 path: unit of length of its FP32 numbers (length_unit)
   md_tuning tun{4, 256, 0.3, 0.7};
   cudaStream_t stream = nullptr;
   int device = 0, nsm = 0;
@@ -403,7 +404,7 @@ struct RdfArgs {
   bool mixed;
   int64_t ntot;
   int nbins, ndim, nrep;
-  double dr, skin;
+  double dr, skin, iunit;  // (iunit: 1 / md_system::unit)
   const RepDev* reps;
   const int32_t* tile_rep;
   const uint4* xbq;   // positions at the last list build: the cells that slots are sorted by
@@ -523,10 +524,10 @@ __device__ __forceinline__ void rdf_scan(const RdfArgs& a, const RepDev& R, RdfW
   }
 }
 
-// Layers of cells that hold the partners within rmax; false: too few cells for
+// Layers of cells that hold the partners within reach (rmax + skin); false: too few cells for
 // that, every slot of the replica is a candidate.
-__device__ __host__ __forceinline__ bool rdf_layers(double rmax, double skin, int nc, float cellw, int* layers) {
-  *layers = nc > 0 ? (int)ceil((rmax + skin) * (1.0 + 1e-6) / (double)cellw) : 0;
+__device__ __host__ __forceinline__ bool rdf_layers(double reach, int nc, float cellw, int* layers) {
+  *layers = nc > 0 ? (int)ceil(reach * (1.0 + 1e-6) / (double)cellw) : 0;
   return nc > 0 && 2 * *layers + 1 <= nc;
 }
 
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(RDF_LIST) k_rdf_units(RdfArgs a) {
   bool first = false;
   int layers;
   if (in && k < R.n) {
-    if (!rdf_layers(a.dr * a.nbins, a.skin, R.nc, R.cellw, &layers)) {
+    if (!rdf_layers((a.dr * a.nbins + a.skin) * a.iunit, R.nc, R.cellw, &layers)) {
       first = k % RDF_PART == 0;
     } else if (k == 0 || i % RDF_CUT == 0) {
       first = true;
@@ -597,17 +598,17 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   if (priv)
     for (int t = threadIdx.x; t < 3 * a.nbins; t += blockDim.x) sh_h[t] = 0u;
   __syncthreads();
-  const double rmax = a.dr * a.nbins;
+  const double dr = a.dr * a.iunit, rmax = dr * a.nbins;  // as the FP32 numbers are
   const int nc = R.nc;
   int layers;
-  const bool all = !rdf_layers(rmax, a.skin, nc, R.cellw, &layers);
+  const bool all = !rdf_layers(rmax + a.skin * a.iunit, nc, R.cellw, &layers);
   const int units = a.nunits[r];
   const bool rel = !all && 2 * (RDF_CELLS + layers + 1) < nc;
   // the FP32 distance is off by less than err: the rounding of coordinates of
   // at most `span`, and the words' own error
   const double span = rel ? (double)(RDF_CELLS + layers + 1) * (double)R.cellw : rmax;
-  const double err = 1e-6 * span + 8.0 * R.L / 4294967296.0;
-  const float edge = (float)(err / a.dr + 1e-6 * a.nbins), invdr = (float)(1.0 / a.dr);
+  const double err = 1e-6 * span + 8.0 * (R.L * a.iunit) / 4294967296.0;
+  const float edge = (float)(err / dr + 1e-6 * a.nbins), invdr = (float)(1.0 / dr);
   const float rmax2f = (float)((rmax + 2.0 * err) * (rmax + 2.0 * err) * (1.0 + 1e-6));
   RdfWarp& W = sh_w[warp];
   int head = 0, count = 0;  // the queue; head also counts the pairs binned since the last flush
@@ -855,8 +856,8 @@ void layout_cells(md_system* s) {
     if (nc < 3) nc = 0;
     R.nc = nc;
     R.nr = nc > 0 ? nr : 1;
-    R.cellw = nc > 0 ? (float)(R.L / nc) : 0.0f;
-    R.mg = s->mixed ? 0.0f : (float)(4.0 * std::sqrt(3.0) * (rl + off) * off);
+    R.cellw = nc > 0 ? (float)(R.L / nc / s->unit) : 0.0f;
+    R.mg = s->mixed ? 0.0f : (float)(4.0 * std::sqrt(3.0) * ((rl + off) / s->unit) * (off / s->unit));
     R.cell0 = cell0;
     R.cs0 = cell0 + r;
     cell0 += (int64_t)nc * nc * nc;
@@ -875,7 +876,7 @@ int list_capacity(const md_system* s) {
   }
   // particles within the list radius: a sphere, or in two dimensions a disc
   double est = s->ndim == 3 ? 4.0 / 3.0 * M_PI * rl * rl * rl * dens : M_PI * rl * rl * dens;
-  int cap = (int)std::ceil(1.5 * est + 32);
+  int cap = (int)std::min(std::ceil(1.5 * est + 32), 1e9);  // (a skin may be many times the box)
   // KAMD_LIST_CAPACITY: start from a given capacity (the list still grows on overflow)
   if (const char* e = std::getenv("KAMD_LIST_CAPACITY")) cap = std::max(1, std::atoi(e));
   if (cap > nmax - 1) cap = (int)std::max<int64_t>(nmax - 1, 1);
@@ -898,7 +899,7 @@ void choose_groups(md_system* s) {
     int g = 1;
     if (R.nc > 0) {
       // particles per occupied cell (two dimensions: only the cells of the plane hold particles)
-      const double w = (double)R.cellw;
+      const double w = (double)R.cellw * s->unit;
       const double occ = s->ndim == 3 ? (double)s->n_per[r] / (R.L * R.L * R.L) * w * w * w
                                       : (double)s->n_per[r] / (R.L * R.L) * w * w;
       // 10 % headroom: a group whose particles overflow the CTA needs a second,
@@ -935,7 +936,7 @@ int stage_capacity(md_system* s) {
     // occupied union cells (two dimensions: one plane of cells)
     const int e = 2 * R.nr;
     const double nu = s->ndim == 3 ? (double)(R.gx + e) * (R.gy + e) * (R.gz + e) : (double)(R.gx + e) * (R.gy + e);
-    const double w = (double)R.cellw;
+    const double w = (double)R.cellw * s->unit;
     const double occ = s->ndim == 3 ? (double)s->n_per[r] / (R.L * R.L * R.L) * w * w * w
                                     : (double)s->n_per[r] / (R.L * R.L) * w * w;
     int need;
@@ -1073,8 +1074,9 @@ void fill_tables(const md_system* s, KParams& p) {
     const double e = s->eps[t], sg = s->sig[t], rc = s->rc[t];
     const double sr6 = std::pow(sg / rc, 6.0);
     const double vc = 4.0 * e * (sr6 * sr6 - sr6);
-    const double rl = rc + s->tun.skin_outer, rli = rc + s->tun.skin;
-    const double s6 = sg * sg * sg * sg * sg * sg;
+    const double u = s->unit;
+    const double rl = (rc + s->tun.skin_outer) / u, rli = (rc + s->tun.skin) / u;
+    const double sgu = sg / u, s6 = sgu * sgu * sgu * sgu * sgu * sgu;
     p.tab_d[t][0] = rc * rc;
     p.tab_d[t][1] = 48.0 * e * s6 * s6;
     p.tab_d[t][2] = 24.0 * e * s6;
@@ -1082,7 +1084,7 @@ void fill_tables(const md_system* s, KParams& p) {
     p.tabe_d[t][0] = 4.0 * e * s6 * s6;
     p.tabe_d[t][1] = 4.0 * e * s6;
     p.rli2_f[t] = (float)(rli * rli * (1.0 + 1e-5));
-    p.rcw2_f[t] = (float)(rc * rc * (1.0 + 1e-5));
+    p.rcw2_f[t] = (float)((rc / u) * (rc / u) * (1.0 + 1e-5));
     p.tab_f[t][0] = (float)(rc * rc);
     p.tab_f[t][1] = (float)(sg * sg);
     p.tab_f[t][2] = (float)(48.0 * e);
@@ -1112,14 +1114,15 @@ KParams make_params(const md_system* s) {
   // inner list once a particle moved skin/2 since the last prune. With
   // skin_outer == skin there is one list: rebuilt at skin/2, never pruned,
   // and the force phase reads it directly
-  const double so = s->tun.skin_outer, si = s->tun.skin;
-  p.dual = so > si ? 1 : 0;
-  p.skin_half2 = p.dual ? 0.25 * (so - si) * (so - si) : 0.25 * si * si;
-  p.prune_half2 = p.dual ? 0.25 * si * si : HUGE_VAL;
+  const double so = s->tun.skin_outer / s->unit, si = s->tun.skin / s->unit;
+  p.dual = s->tun.skin_outer > s->tun.skin ? 1 : 0;
+  p.skin_half2f = (float)(p.dual ? 0.25 * (so - si) * (so - si) : 0.25 * si * si);
+  p.prune_half2f = p.dual ? (float)(0.25 * si * si) : (float)HUGE_VAL;
+  p.scaled = s->unit != 1.0 ? 1 : 0;
+  p.unit2 = s->unit * s->unit;
+  p.iunit2 = 1.0 / p.unit2;
   p.massf = (float)s->mass;
   p.inv_massf = (float)(1.0 / s->mass);
-  p.skin_half2f = (float)p.skin_half2;
-  p.prune_half2f = (float)p.prune_half2;
   p.timeout_ns = s->timeout_ns;
   p.reps = s->d_reps;
   p.tile_rep = s->d_tile_rep;
@@ -1447,6 +1450,7 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
     s->sig[t] = sigma[t];
     s->rc[t] = rc[t];
   }
+  if (!s->mixed) s->unit = length_unit(rc_max(s));
   if (const char* e = std::getenv("KAMD_BARRIER_TIMEOUT_MS")) s->timeout_ns = (unsigned long long)std::atoll(e) * 1000000ull;
   if (const char* e = std::getenv("KAMD_NO_GRAPH")) s->use_graph = !(e[0] == '1');
   if (const char* e = std::getenv("KAMD_LOG_NOW")) s->log_now = e[0] == '1';
@@ -1480,7 +1484,7 @@ md_status md_create_batch_dim(int ndim, int nrep, const int64_t* n_per, const do
     R.invL = 1.0 / L_per[r];
     R.fx64 = 18446744073709551616.0 / L_per[r];
     R.Lf = (float)L_per[r];
-    R.fxs = (float)(L_per[r] / 4294967296.0);
+    R.fxs = (float)(L_per[r] / 4294967296.0 / s->unit);
     R.fx64f = (float)R.fx64;
     R.fx32f = (float)(4294967296.0 / L_per[r]);
     R.fx32 = 4294967296.0 / L_per[r];
@@ -1758,6 +1762,7 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
   a.nrep = s->nrep;
   a.dr = dr;
   a.skin = s->tun.skin_outer;
+  a.iunit = 1.0 / s->unit;
   a.reps = s->d_reps;
   a.tile_rep = s->d_tile_rep;
   a.xbq = s->d_xbq;
@@ -1780,7 +1785,7 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
     const RepDev& R = s->reps[r];
     int l;
     double share = 0.5;
-    if (rdf_layers(dr * nbins, a.skin, R.nc, R.cellw, &l))
+    if (rdf_layers((dr * nbins + a.skin) * a.iunit, R.nc, R.cellw, &l))
       share = std::min(0.5, (2.0 * l + RDF_CELLS) * (l + 1.0) * (s->ndim == 3 ? 2.0 * l + 1.0 : 1.0) /
                                 std::pow((double)R.nc, (double)s->ndim));
     work[r] = (double)R.n * (double)R.n * share;
@@ -2090,7 +2095,7 @@ md_status md_count_pairs(md_system* s, int64_t* pairs) {
   CK(cudaMemsetAsync(s->d_count, 0, 8, s->stream));
   const int b = 128;
   k_count_pairs<<<blocks_for(s->ntot, b), b, 0, s->stream>>>(
-      s->mixed, s->ntot, s->ntypes, rc_max(s) + s->tun.skin_outer, s->d_reps, s->d_tile_rep, s->d_pfx,
+      s->mixed, s->ntot, s->ntypes, (rc_max(s) + s->tun.skin_outer) / s->unit, s->d_reps, s->d_tile_rep, s->d_pfx,
       s->d_p4[s->ctl.cur], s->d_typ, s->d_cstart, s->d_io, s->d_count);
   CK(cudaGetLastError());
   unsigned long long c = 0;

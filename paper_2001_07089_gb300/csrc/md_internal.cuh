@@ -24,6 +24,7 @@
 // the natural overflow of the integer; the minimum-image difference of two
 // particles is the signed 32-bit difference of their top words, exact.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <cuda_runtime.h>
@@ -62,11 +63,11 @@ struct RepDev {
   int32_t gx, gy, gz;  // cells per list-build group along x, y, z (1, 2 or 4 each; per replica)
   double L, invL;
   double fx64;      // 2^64 / L
-  float Lf, fxs;    // L, L / 2^32
+  float Lf, fxs;    // L, and L / 2^32 in units of md_system::unit
   float fx64f;      // 2^64 / L
   float fx32f;      // 2^32 / L
-  float cellw;      // L / nc
-  float mg;         // FP64 path: bound on the error of a squared distance taken from 32-bit words (mixed: 0)
+  float cellw;      // L / nc, in that unit
+  float mg;         // FP64 path (same unit): bound on the error of a squared distance taken from 32-bit words (mixed: 0)
   double fx32;      // 2^32 / L
   // bath
   double T_target, Q;
@@ -144,12 +145,16 @@ struct KParams {
   float rl2_f[MD_MAXTYPES * MD_MAXTYPES];      // outer list radius^2: (rc + skin_outer)^2
   float rli2_f[MD_MAXTYPES * MD_MAXTYPES];     // inner list radius^2: (rc + skin)^2
   float rcw2_f[MD_MAXTYPES * MD_MAXTYPES];     // rc^2, widened: the FP64 path's pre-test
-  double tab_d[MD_MAXTYPES * MD_MAXTYPES][4];  // rc^2, 48 eps sigma^12, 24 eps sigma^6, V(rc)
+  double tab_d[MD_MAXTYPES * MD_MAXTYPES][4];  // rc^2 (as given), 48 eps sigma^12, 24 eps sigma^6, V(rc)
   double tabe_d[MD_MAXTYPES * MD_MAXTYPES][2]; // 4 eps sigma^12, 4 eps sigma^6
+  // FP64 path: the squares of lists, margins and triggers, and sigma in the table, are in a unit of
+  // length other than 1 if `scaled` (see length_unit); its square and that square's inverse
+  int scaled;
+  double unit2, iunit2;
   double mass, inv_mass;
-  double skin_half2;   // ((skin_outer - skin)/2)^2, one list: (skin/2)^2: move since the build that forces a rebuild
-  double prune_half2;  // (skin/2)^2, one list: infinite: move since the last prune that forces a prune
-  float massf, inv_massf, skin_half2f, dtf, prune_half2f;
+  float massf, inv_massf, dtf;
+  float skin_half2f;   // ((skin_outer - skin)/2)^2, one list: (skin/2)^2: move since the build that forces a rebuild
+  float prune_half2f;  // (skin/2)^2, one list: infinite: move since the last prune that forces a prune
   // operation
   int op;
   int kind;
@@ -216,6 +221,15 @@ struct KParams {
   int64_t plog_stride;
   int plog_slots;
 };
+
+// Unit of length of the FP32 numbers of an FP64 path with the largest cutoff rc:
+// 1 for anything like usual, else the power of two at rc, so that the squares of
+// lengths (and the powers of sigma, in FP64) stay far from the ends of the range
+// whatever the caller's unit. Powers of two: no rounding.
+inline double length_unit(double rc) {
+  const int k = std::ilogb(rc);
+  return k < -40 || k > 40 ? std::ldexp(1.0, k) : 1.0;
+}
 
 // Host-side launchers (md_kernel.cu).
 cudaError_t md_launch_persistent(bool mixed, const KParams& p, int grid, int block, size_t smem, int carveout,

@@ -399,17 +399,20 @@ __device__ __forceinline__ void lane_sum_mix(const Shared& sh, const uint4* __re
 // Pair term for one list entry (FP64 path), Eq. (KAFix) and Eq. (VshiftedKALJ)
 // with sigma folded into the constants (16 FP64 operations without energy, 12
 // of them FMAs or multiplies of the pair itself).
-template <bool ENERGY>
-__device__ __forceinline__ void pair_f64(const Shared& sh, const double4_32a& pi, const double4_32a& pj, int tt, double L,
+// SCALED: sigma is in another unit of length than the positions (p.scaled).
+template <bool ENERGY, bool SCALED>
+__device__ __forceinline__ void pair_f64(const KParams& p, const Shared& sh, const double4_32a& pi, const double4_32a& pj, int tt, double L,
                                          long long hLb, double& fx, double& fy, double& fz, double& pe, double& vir) {
   const double dx = image_f64(pi.x - pj.x, L, hLb), dy = image_f64(pi.y - pj.y, L, hLb), dz = image_f64(pi.z - pj.z, L, hLb);
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
   const double4_32a c = sh.tabd[tt];
   if (less_f64(r2, c.x)) {
-    const double y = rcp_f64(r2);
+    double y = rcp_f64(r2);
+    if (SCALED) y *= p.unit2;
     const double y3 = y * y * y;
     const double w = y3 * fma(c.y, y3, -c.z);
-    const double fr = w * y;
+    double fr = w * y;
+    if (SCALED) fr *= p.iunit2;
     fx = fma(fr, dx, fx);
     fy = fma(fr, dy, fy);
     fz = fma(fr, dz, fz);
@@ -479,7 +482,10 @@ __device__ __forceinline__ void unit_sum_f64(const KParams& p, const Shared& sh,
       const int q = 4 * row0 + (e >> tsh);  // place in the column of lane e % T
       const int jj = lp[list_at(4 * ((e & (T - 1)) - s), q, gsz)];
       const double4_32a pj4 = p4[jj];
-      pair_f64<ENERGY>(sh, pi, pj4, tb + __double2loint(pj4.w), L, hLb, fx, fy, fz, pe, vir);
+      const int tt = tb + __double2loint(pj4.w);
+      // (one branch: two multiplications under a condition took 6 % of the step)
+      if (__builtin_expect(p.scaled, 0)) pair_f64<ENERGY, true>(p, sh, pi, pj4, tt, L, hLb, fx, fy, fz, pe, vir);
+      else pair_f64<ENERGY, false>(p, sh, pi, pj4, tt, L, hLb, fx, fy, fz, pe, vir);
     }
     __syncwarp();
     held = 0;

@@ -56,10 +56,13 @@ constexpr size_t kScratchBytes = (kOffTicket + 256 + 255) / 256 * 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 struct Table {
-  // rc^2, 48 eps sigma^12, 24 eps sigma^6, 4 eps sigma^12, 4 eps sigma^6, V(rc); rc^2 widened, FP32
+  // rc^2 (as given), 48 eps sigma^12, 24 eps sigma^6, 4 eps sigma^12, 4 eps sigma^6, V(rc); rc^2 widened, FP32:
+  // sigma and the last in units of length_unit(), whose square and its inverse are used if it is not 1
   double rc2[kMaxTypes * kMaxTypes], c12[kMaxTypes * kMaxTypes], c6[kMaxTypes * kMaxTypes], e12[kMaxTypes * kMaxTypes],
       e6[kMaxTypes * kMaxTypes], vsh[kMaxTypes * kMaxTypes];
   float rcw2[kMaxTypes * kMaxTypes];
+  int scaled;
+  double unit, unit2, iunit2;
 };
 
 struct Scratch {
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(Scratch s, const doubl
   for (int t = tid; t < (int)(sizeof(Table) / 4); t += kForceThreads)
     reinterpret_cast<int*>(&tb)[t] = reinterpret_cast<const int*>(&tab)[t];
   const double to_word = 4294967296.0 / L;
-  const float sc = (float)(L / 4294967296.0);
+  const float sc = (float)(L / 4294967296.0 / tab.unit);
   const long long hLb = __double_as_longlong(0.5 * L);
   double pe = 0.0, vir = 0.0;
   const int items = nc > 0 ? *s.nitems : (n + kItem - 1) / kItem;
@@ -325,10 +328,12 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(Scratch s, const doubl
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
             const int tt = row + min((int)(word[h].w >> 30), ntypes - 1);
             if (kamd::less_f64(r2, tb.rc2[tt])) {
-              const double y = kamd::rcp_f64(r2);
+              double y = kamd::rcp_f64(r2);
+              if (__builtin_expect(tab.scaled, 0)) y *= tab.unit2;
               const double y3 = y * y * y;
               const double w = y3 * fma(tb.c12[tt], y3, -tb.c6[tt]);
-              const double fr = w * y;
+              double fr = w * y;
+              if (__builtin_expect(tab.scaled, 0)) fr *= tab.iunit2;
               fx = fma(fr, dx, fx);
               fy = fma(fr, dy, fy);
               fz = fma(fr, dz, fz);
@@ -491,19 +496,23 @@ extern "C" md_status md_forces_noalloc(int64_t n, const double* pos, const uint8
         return noalloc_fail(MD_ERR_INVALID_ARG, "md_forces_noalloc: tables must be positive and symmetric");
       if (!(rc[t] < 0.5 * L)) return noalloc_fail(MD_ERR_INVALID_ARG, "md_forces_noalloc: every cutoff must be < L/2");
       const double sr6 = std::pow(sigma[t] / rc[t], 6.0);
-      const double s3 = sigma[t] * sigma[t] * sigma[t], s6 = s3 * s3;
       tab.rc2[t] = rc[t] * rc[t];
-      tab.c12[t] = 48.0 * eps[t] * s6 * s6;
-      tab.c6[t] = 24.0 * eps[t] * s6;
-      tab.e12[t] = 4.0 * eps[t] * s6 * s6;
-      tab.e6[t] = 4.0 * eps[t] * s6;
       tab.vsh[t] = 4.0 * eps[t] * (sr6 * sr6 - sr6);
       rcmax = std::max(rcmax, rc[t]);
     }
   // the FP32 pre-test: r^2 from 32-bit words is off by less than 4 r sqrt(3) L/2^31 and a relative 1e-6
-  const double off = std::ldexp(L, -31);
-  for (int t = 0; t < ntypes * ntypes; ++t)
-    tab.rcw2[t] = (float)(rc[t] * rc[t] * (1.0 + 1e-5) + 4.0 * std::sqrt(3.0) * (rc[t] + off) * off);
+  const double u = tab.unit = length_unit(rcmax), off = std::ldexp(L, -31) / u;
+  tab.scaled = u != 1.0;
+  tab.unit2 = u * u;
+  tab.iunit2 = 1.0 / tab.unit2;
+  for (int t = 0; t < ntypes * ntypes; ++t) {
+    const double s1 = sigma[t] / u, s3 = s1 * s1 * s1, s6 = s3 * s3, r = rc[t] / u;
+    tab.c12[t] = 48.0 * eps[t] * s6 * s6;
+    tab.c6[t] = 24.0 * eps[t] * s6;
+    tab.e12[t] = 4.0 * eps[t] * s6 * s6;
+    tab.e6[t] = 4.0 * eps[t] * s6;
+    tab.rcw2[t] = (float)(r * r * (1.0 + 1e-5) + 4.0 * std::sqrt(3.0) * (r + off) * off);
+  }
   // cells of edge >= the largest cutoff, at most kMaxCellsPerEdge per edge
   // (clamped in double, so any finite L is safe); fewer than 3: all pairs
   int nc = (int)std::min(std::floor(L / rcmax), (double)kMaxCellsPerEdge);

@@ -1,5 +1,5 @@
 """The FP64 force paths (md_forces of an FP64 system and md_forces_noalloc) on inputs that their FP32 tests and
-bit-pattern comparisons have to carry: positions that are not numbers, particles in one place."""
+bit-pattern comparisons have to carry: positions that are not numbers, particles in one place, any unit of length."""
 import numpy as np
 import pytest
 
@@ -75,3 +75,30 @@ def test_particles_in_one_place():
     for f, pe, w in results:
         assert pe == np.inf and w == np.inf
         assert np.all(np.isnan(f[two])) and force_errors(f[~two], f_ref)[0] <= 1e-11
+
+
+@pytest.mark.parametrize("power", [-300, -70, -41, 41, 70, 300])
+def test_any_unit_of_length(power):
+    """Lengths in units of 2^power: their squares leave the range of FP32 (and sigma^12 that of FP64). Energies,
+    virials and g(r) are those of power 0, forces and positions scale, in single calls and over steps."""
+    pos, vel, types, L = melted(1000, 22, nsteps=200)
+    f1, pe1, w1 = noalloc(pos, types, L)
+
+    def run(u, skin):
+        with kamd.System(1000, L * u, types, wl.KA_EPS, wl.KA_SIG * u, wl.KA_RC * u, u ** -2.0, skin, "fp64") as s:
+            s.set_tuning(skin=skin, skin_outer=skin)
+            s.set_state(pos * u, vel * u)
+            f, pe, w = s.forces()
+            log = s.step_nve(0.004, 20, log_every=10)
+            g = s.rdf(0.02 * u, 200, reset=True)
+            p, v, img = s.get_state()
+            return f * u, pe, w, p / u, v / u, img, g, log["pe_per_n"], log["T"], s.count_pairs(), s.msd() / u ** 2
+
+    u = 2.0 ** power
+    f, pe, w = noalloc(pos * u, types, L * u, wl.KA_EPS, wl.KA_SIG * u, wl.KA_RC * u)
+    assert force_errors(f * u, f1)[0] <= 1e-12 and abs(pe - pe1) <= 1e-12 * abs(pe1) and abs(w - w1) <= 1e-11 * abs(w1)
+    # (a skin beyond 2 is refused, and a skin of 0.3 at large lengths is next to none)
+    a, b = run(1.0, 0.3), run(u, 0.3 * min(u, 1.0))
+    assert force_errors(b[0], a[0])[0] <= 1e-12
+    for x, y in zip(b[1:], a[1:]):
+        assert np.allclose(x, y, rtol=1e-9, atol=1e-9), (x, y)
