@@ -857,7 +857,14 @@ void layout_cells(md_system* s) {
     R.nc = nc;
     R.nr = nc > 0 ? nr : 1;
     R.cellw = nc > 0 ? (float)(R.L / nc / s->unit) : 0.0f;
-    R.mg = s->mixed ? 0.0f : (float)(4.0 * std::sqrt(3.0) * ((rl + off) / s->unit) * (off / s->unit));
+    // Margin of the FP64 path's squared distances from 32-bit words. Per coordinate,
+    // a difference of words is off by off/2; the list build's differences of FP32
+    // coordinates, up to four cells from the group's first particle, by another
+    // 1.5 off in the widest cells (1024 per edge; in narrower ones the tests'
+    // relative 1e-5 holds that); and two particles may each have moved off/2 more
+    // than the triggers see: 3 off in all, taken as 4
+    const double err = 4.0 * std::sqrt(3.0) * off / s->unit;
+    R.mg = s->mixed ? 0.0f : (float)((2.0 * rl / s->unit + err) * err);
     R.cell0 = cell0;
     R.cs0 = cell0 + r;
     cell0 += (int64_t)nc * nc * nc;
