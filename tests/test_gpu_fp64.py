@@ -102,3 +102,27 @@ def test_any_unit_of_length(power):
     assert force_errors(b[0], a[0])[0] <= 1e-12
     for x, y in zip(b[1:], a[1:]):
         assert np.allclose(x, y, rtol=1e-9, atol=1e-9), (x, y)
+
+
+def test_reciprocal_in_the_pair_term():
+    """32 768 pairs alone in their cells, at r^2 over the cutoff's range and beside powers of two. With u = 2^-53:
+    1/r^2 is off by at most 2 u (r^2 and the reciprocal rounded), its cube by 8 u, the two terms of the bracket
+    by 16 + 6 and 8 + 5 u (sigma and epsilon are 1), the product with 1/r^2 and r by 4 u more."""
+    n, L, cell = 32768, 256.0, 8.0
+    rng = np.random.default_rng(12)
+    r = rng.uniform(0.72, 2.49, n)
+    near = np.sqrt(2.0 ** rng.integers(-1, 3, n // 4) * (1 + rng.integers(-8, 9, n // 4) * 2.0 ** -44))
+    r[:n // 4] = np.clip(near, 0.72, 2.49)
+    a = np.stack(np.unravel_index(np.arange(n), (32,) * 3), 1) * cell + 2.0
+    axis = np.arange(n) % 3
+    b = a.copy()
+    b[np.arange(n), axis] += r
+    d = (b - a)[np.arange(n), axis].astype(np.longdouble)  # exact: both are multiples of 2^-45
+    one = np.ones((1, 1))
+    f, _, _ = noalloc(np.concatenate([a, b]), np.zeros(2 * n), L, one, one, 2.5 * one)
+    got = f[n + np.arange(n), axis].astype(np.longdouble)
+    y = 1 / (d * d)
+    attract, repel = 24 * y ** 3, 48 * y ** 6
+    bound = 32 * np.longdouble(2) ** -53 * (repel + attract) * y * d
+    assert np.all(np.abs(got - (repel - attract) * y * d) <= bound)
+    assert np.array_equal(f[:n], -f[n:])
