@@ -268,7 +268,8 @@ md_status md_get_tuning(const md_system* sys, md_tuning* t);
  * md_autotune: time short NVE probes (probe_steps each, dt) and keep the
  * fastest candidate. Coordinate search: threads_per_atom x block_size at the
  * current skins, then nine (skin, skin_outer) pairs (three of them one-list)
- * at the best of those, then threads_per_atom x block_size at the best pair.
+ * at the best of those, then threads_per_atom x block_size at the best pair
+ * (threads_per_atom of an FP64 system: 4 and 8, since it has no fewer).
  * The system's state is saved before and restored after, so the trajectory
  * is unaffected. best (may be NULL) receives the choice, seconds_per_step (may
  * be NULL) its measured cost.

@@ -1908,6 +1908,8 @@ static md_status autotune_impl(md_system* s, double dt, int64_t probe_steps, dou
   auto probe = [&](const md_tuning& c) {
     if (st != MD_OK) return;
     if (c.block_size < 32 * c.threads_per_atom) return;
+    // fewer lanes than the lists get: the same program as more (see list_lanes)
+    if (!s->mixed && c.threads_per_atom < 4) return;
     if (tuning_ok(s, &c) != MD_OK) return;
     st = md_set_tuning(s, &c);
     if (st == MD_OK) st = set_state_impl(s, saved, saved + n3, 1);

@@ -77,6 +77,18 @@ def test_particles_in_one_place():
         assert np.all(np.isnan(f[two])) and force_errors(f[~two], f_ref)[0] <= 1e-11
 
 
+def test_autotune_names_the_lanes_that_run():
+    """An FP64 system has at least four lanes per particle: fewer are the same program, and are not tried."""
+    n = 256
+    L = wl.box_length(n)
+    with kamd.System(n, L, wl.ka_types(n, 3).astype(np.int32), wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3, "fp64") as s:
+        s.set_tuning(threads_per_atom=1, block_size=256, skin=0.3, skin_outer=0.3)
+        s.init_lattice(0.5, seed=5)
+        for skin in (None, 0.25):
+            tun, _ = s.autotune(0.004, probe_steps=4, skin=skin)
+            assert tun["threads_per_atom"] >= 4 and s.tuning["threads_per_atom"] >= 4, tun
+
+
 @pytest.mark.parametrize("power", [-300, -70, -41, 41, 70, 300])
 def test_any_unit_of_length(power):
     """Lengths in units of 2^power: their squares leave the range of FP32 (and sigma^12 that of FP64). Energies,
