@@ -12,6 +12,17 @@
 #include "md_device.cuh"
 #include "md_internal.cuh"
 
+// A shape of the persistent launch, and the launch as an instantiated CUDA graph
+// (one cooperative kernel node whose parameters are updated per call).
+struct LaunchShape {
+  int grid = 0, carveout = 0;  // CTAs; percent of the SM's shared memory that they take
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t gexec = nullptr;
+  cudaGraphNode_t gnode = nullptr;
+  int g_grid = 0, g_block = 0, g_carveout = 0;
+  size_t g_smem = 0;
+};
+
 struct md_system {
   // configuration
   int nrep = 0, ntypes = 0;
@@ -29,7 +40,6 @@ struct md_system {
   md_tuning tun{4, 256, 0.3, 0.7};
   cudaStream_t stream = nullptr;
   int device = 0, nsm = 0;
-  int grid = 0;
   int maxrows = 0;
   int stage_cap = 0;  // candidates the list build stages per group (dynamic shared memory)
   int64_t ncells = 0;
@@ -104,8 +114,7 @@ struct md_system {
   std::unordered_map<const void*, size_t> alloc_sizes;
   size_t list_bytes = 0;
   unsigned long long timeout_ns = 10ull * 1000 * 1000 * 1000;
-  // the persistent launch as an instantiated CUDA graph (one cooperative
-  // kernel node whose parameters are updated per call)
+  LaunchShape shape[2];  // the usual one, and the one of as many CTAs as fit (configure_grid, wide_launch)
   bool use_graph = true;
   // partial records of NVE log steps reduced after the launch (size in doubles)
   double* d_plog = nullptr;
@@ -113,12 +122,6 @@ struct md_system {
   size_t plog_cap = 0;
   int plog_slots = 0;
   bool log_now = false;  // KAMD_LOG_NOW=1: every log record reduced at its step
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t gexec = nullptr;
-  cudaGraphNode_t gnode = nullptr;
-  int g_grid = 0, g_block = 0;
-  size_t g_smem = 0;
-  int carveout = 0, g_carveout = 0;  // percent of the SM's shared memory that the grid takes
   int64_t graph_launches = 0;
   int64_t kernel_launches = 0;  // persistent launches and log-record launches
   std::string err;
@@ -1058,19 +1061,23 @@ md_status configure_grid(md_system* s) {
   int groups = 0;
   for (const auto& R : s->reps) groups = std::max(groups, R.ngrp);
   const bool small = groups <= s->nsm && (int64_t)s->ntiles * list_lanes(s) <= (int64_t)s->nsm * (b / 32);
-  s->grid = (small ? 1 : per_sm) * s->nsm;
-  // The split between shared memory and L1 is asked for at each launch: no more
-  // shared memory than the resident CTAs take, since the force phase's gathers
-  // live in L1. The driver's own choice was larger: N = 10^6, force phase 199 ->
-  // 191 us; 20 steps of N = 8*10^6 56.3 -> 54.0 ms. (A launch attribute: other
-  // systems of the process have other needs.)
-  CK(md_carveout(s->mixed, stage_bytes(s), small ? 1 : per_sm, &s->carveout));
-  if (s->grid > s->cta_sm_cap) {
+  for (int w = 0; w < 2; ++w) {
+    const int n = w == 0 && small ? 1 : per_sm;
+    s->shape[w].grid = n * s->nsm;
+    // The split between shared memory and L1 is asked for at each launch: no more
+    // shared memory than the resident CTAs take, since the force phase's gathers
+    // live in L1. The driver's own choice was larger: N = 10^6, force phase 199 ->
+    // 191 us; 20 steps of N = 8*10^6 56.3 -> 54.0 ms. (A launch attribute: other
+    // systems of the process have other needs.)
+    CK(md_carveout(s->mixed, stage_bytes(s), n, &s->shape[w].carveout));
+  }
+  const int most = s->shape[1].grid;
+  if (most > s->cta_sm_cap) {
     dfree(s, s->d_cta_sm);
     s->d_cta_sm = nullptr;
     s->cta_sm_cap = 0;
-    CKS(dalloc(s, &s->d_cta_sm, (size_t)s->grid));
-    s->cta_sm_cap = s->grid;
+    CKS(dalloc(s, &s->d_cta_sm, (size_t)most));
+    s->cta_sm_cap = most;
   }
   return MD_OK;
 }
@@ -1184,19 +1191,37 @@ KParams make_params(const md_system* s) {
   return p;
 }
 
-void drop_graph(md_system* s) {
-  if (s->gexec) cudaGraphExecDestroy(s->gexec);
-  if (s->graph) cudaGraphDestroy(s->graph);
-  s->gexec = nullptr;
-  s->graph = nullptr;
-  s->gnode = nullptr;
+void drop_graph(LaunchShape& h) {
+  if (h.gexec) cudaGraphExecDestroy(h.gexec);
+  if (h.graph) cudaGraphDestroy(h.graph);
+  h.gexec = nullptr;
+  h.graph = nullptr;
+  h.gnode = nullptr;
+}
+
+// Whether a launch takes as many CTAs as fit although one per SM holds each
+// replica's groups: when replicas that rebuild together have more groups than
+// there are SMs, and the steps that follow are too few to repay the wait for
+// them with cheaper barriers. Measured on 8 replicas of 1000 that all rebuild
+// (216 groups), T = 4 and 256 threads, 152 CTAs against 608: forces 185 and 137
+// us, NVE of 20 steps 525 and 488, of 40 1128 and 1140; Nose-Hoover of 20 682 and
+// 644, of 50 1679 and 1727; resampling of 50 829 and 1027; FP64 on 456 CTAs,
+// 10 steps 672 and 662, of 20 1310 and 1314.
+bool wide_launch(const md_system* s, int op, int kind, int64_t nsteps) {
+  if (s->shape[0].grid == s->shape[1].grid || !(s->ctl.pending & MD_FLAG_REBUILD)) return false;
+  if (!s->reps_now && !s->reps_dirty) return false;  // not known here
+  if (op == MD_OP_FORCE_REPEAT || op == MD_OP_LIST_REPEAT) return false;
+  int64_t groups = 0;
+  for (const auto& R : s->reps) groups += R.want_rebuild ? R.ngrp : 0;
+  const int64_t few = s->mixed && kind != MD_KIND_RESAMPLE ? 24 : 10;
+  return groups > s->shape[0].grid && (op != MD_OP_STEPS || nsteps <= few);
 }
 
 // Launch the persistent kernel. By default through an instantiated CUDA graph
 // holding one cooperative kernel node (built once per launch shape, its
 // parameters updated per call); a direct cooperative launch if the graph
 // cannot be built or KAMD_NO_GRAPH is set.
-cudaError_t launch_persistent(md_system* s, const KParams& p) {
+cudaError_t launch_persistent(md_system* s, const KParams& p, LaunchShape& h) {
   const size_t smem = stage_bytes(s);
   const int block = s->tun.block_size;
   if (s->use_graph) {
@@ -1204,48 +1229,47 @@ cudaError_t launch_persistent(md_system* s, const KParams& p) {
     void* args[] = {(void*)&pc};
     cudaKernelNodeParams kp = {};
     kp.func = (void*)md_persistent_fn(s->mixed);
-    kp.gridDim = dim3(s->grid);
+    kp.gridDim = dim3(h.grid);
     kp.blockDim = dim3(block);
     kp.sharedMemBytes = (unsigned)smem;
     kp.kernelParams = args;
     cudaError_t e = cudaSuccess;
-    if (!s->gexec || s->g_grid != s->grid || s->g_block != block || s->g_smem != smem ||
-        s->g_carveout != s->carveout) {
-      drop_graph(s);
+    if (!h.gexec || h.g_grid != h.grid || h.g_block != block || h.g_smem != smem || h.g_carveout != h.carveout) {
+      drop_graph(h);
       e = cudaFuncSetAttribute(kp.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) e = cudaGraphCreate(&s->graph, 0);
-      if (e == cudaSuccess) e = cudaGraphAddKernelNode(&s->gnode, s->graph, nullptr, 0, &kp);
+      if (e == cudaSuccess) e = cudaGraphCreate(&h.graph, 0);
+      if (e == cudaSuccess) e = cudaGraphAddKernelNode(&h.gnode, h.graph, nullptr, 0, &kp);
       if (e == cudaSuccess) {
         cudaKernelNodeAttrValue v = {};
         v.cooperative = 1;
-        e = cudaGraphKernelNodeSetAttribute(s->gnode, cudaKernelNodeAttributeCooperative, &v);
+        e = cudaGraphKernelNodeSetAttribute(h.gnode, cudaKernelNodeAttributeCooperative, &v);
         if (e == cudaSuccess) {
           cudaKernelNodeAttrValue c = {};
-          c.sharedMemCarveout = (unsigned)s->carveout;
-          e = cudaGraphKernelNodeSetAttribute(s->gnode, cudaKernelNodeAttributePreferredSharedMemoryCarveout, &c);
+          c.sharedMemCarveout = (unsigned)h.carveout;
+          e = cudaGraphKernelNodeSetAttribute(h.gnode, cudaKernelNodeAttributePreferredSharedMemoryCarveout, &c);
         }
       }
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&s->gexec, s->graph, 0);
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&h.gexec, h.graph, 0);
       if (e == cudaSuccess) {
-        s->g_grid = s->grid;
-        s->g_block = block;
-        s->g_smem = smem;
-        s->g_carveout = s->carveout;
+        h.g_grid = h.grid;
+        h.g_block = block;
+        h.g_smem = smem;
+        h.g_carveout = h.carveout;
       }
     } else {
-      e = cudaGraphExecKernelNodeSetParams(s->gexec, s->gnode, &kp);
+      e = cudaGraphExecKernelNodeSetParams(h.gexec, h.gnode, &kp);
     }
-    if (e == cudaSuccess) e = cudaGraphLaunch(s->gexec, s->stream);
+    if (e == cudaSuccess) e = cudaGraphLaunch(h.gexec, s->stream);
     if (e == cudaSuccess) {
       ++s->graph_launches;
       return cudaSuccess;
     }
     // the driver refused the graph: clear the error and launch directly from now on
     cudaGetLastError();
-    drop_graph(s);
+    drop_graph(h);
     s->use_graph = false;
   }
-  return md_launch_persistent(s->mixed, p, s->grid, block, smem, s->carveout, s->stream);
+  return md_launch_persistent(s->mixed, p, h.grid, block, smem, h.carveout, s->stream);
 }
 
 // Run the persistent kernel for one operation, growing the neighbour list
@@ -1258,6 +1282,7 @@ md_status run_op(md_system* s, int op, int kind, double dt, int64_t nsteps, int6
     // host mirror is current: every launch ends with a download of it)
     s->ctl.pending &= MD_FLAG_REBUILD;
     s->ctl.err_where = 0;
+    LaunchShape& shape = s->shape[wide_launch(s, op, kind, nsteps - done) ? 1 : 0];
     CKS(upload_state(s));
     KParams p = make_params(s);
     p.op = op;
@@ -1272,7 +1297,7 @@ md_status run_op(md_system* s, int op, int kind, double dt, int64_t nsteps, int6
     p.log_cap = log_cap;
     p.thermo = s->d_thermo;
     s->ctl_now = s->reps_now = false;
-    CK(launch_persistent(s, p));
+    CK(launch_persistent(s, p, shape));
     ++s->kernel_launches;
     CKS(download_state(s, s->nrep <= LAND_REPS));
     if (op == MD_OP_STEPS) done += s->ctl.steps_done;
@@ -2067,7 +2092,7 @@ md_status md_get_info(md_system* s, md_info* info) {
   std::memset(info, 0, sizeof(*info));
   info->n_total = s->n_total;
   info->n_replicas = s->nrep;
-  info->grid_blocks = s->grid;
+  info->grid_blocks = s->shape[0].grid;
   info->steps_done = s->ctl.step;
   for (const auto& R : s->reps) {
     info->rebuilds += R.rebuilds;
@@ -2156,7 +2181,7 @@ const char* md_last_error(const md_system* s) {
 void md_destroy(md_system* s) {
   if (!s) return;
   if (s->stream) cudaStreamSynchronize(s->stream);
-  drop_graph(s);
+  for (auto& h : s->shape) drop_graph(h);
   if (s->h_land) cudaFreeHost(s->h_land);
   dfree(s, s->d_state); dfree(s, s->d_tile_rep);
   dfree(s, s->d_pfx); dfree(s, s->d_pq[0]); dfree(s, s->d_pq[1]); dfree(s, s->d_velf); dfree(s, s->d_frcf); dfree(s, s->d_xbq);

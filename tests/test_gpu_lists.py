@@ -92,6 +92,33 @@ def test_partial_rebuilds_of_more_replicas_than_threads(prec, block):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_few_replicas_rebuilding_together_equal_their_own_runs(prec):
+    """Eight replicas have more list-build groups than there are SMs but work enough for one CTA per SM: short
+    launches that begin with all their rebuilds take more CTAs, long ones do not. Both are bitwise the same."""
+    n, nrep, L = 1000, 8, wl.box_length(1000)
+    types = [wl.ka_types(n, 30 + k).astype(np.int32) for k in range(nrep)]
+
+    def run(k, cuts):
+        t = np.concatenate(types) if k is None else types[k]
+        m = nrep if k is None else 1
+        with kamd.System([n] * m if m > 1 else n, [L] * m if m > 1 else L, t, wl.KA_EPS, wl.KA_SIG, wl.KA_RC, 1.0, 0.3,
+                         prec) as s:
+            s.init_lattice([1.2] * m if m > 1 else 1.2, seed=19)
+            f = s.forces()[0]
+            for c in cuts:
+                p, v, _ = s.get_state()
+                s.set_state(p, v)  # (every replica rebuilds)
+                s.step_nve(0.004, c)
+            return s.get_state()[:2] + (f, s.forces()[0])
+
+    for cuts in ((8, 60, 8, 60), (60, 8)):
+        x = run(None, cuts)
+        for k in (0, 3, 7):
+            y = run(k, cuts)
+            assert all(np.array_equal(a, b[k * n:(k + 1) * n]) for a, b in zip(y, x)), (cuts, k)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_thousands_of_replicas_equal_their_own_runs(prec):
     """2500 replicas, some with cells and some without, cold and hot, so that any of them rebuild together:
     each is found among the others (bitwise its stand-alone run), and their energies come back."""
