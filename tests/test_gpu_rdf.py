@@ -148,3 +148,22 @@ def test_dilute_boxes_and_droplets(prec, ndim, L):
     c, r = np.rint(g * w), np.rint(ref * w)
     assert r.sum() > 10 * n and np.max(np.abs(g * w - c)) < 1e-6
     assert np.array_equal(c, r)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_uneven_batch_many_bins_and_accumulation(prec):
+    """Replicas of 6000, 20 and 700 particles, more bins than a CTA keeps counts for, after steps: the mean of the
+    replicas' counts is the oracle's; a second call without reset leaves g(r) as it is, another dr starts anew."""
+    ns = [6000, 20, 700]
+    Ls = [wl.box_length(6000), 9.0, wl.box_length(700)]
+    types = [wl.ka_types(n, 40 + k).astype(np.int32) for k, n in enumerate(ns)]
+    off = np.concatenate([[0], np.cumsum(ns)])
+    with system(ns, Ls, np.concatenate(types), prec) as s:
+        s.init_lattice([1.0, 0.3, 2.0], seed=21)
+        s.step_nve(0.004, 30)
+        p, _, _ = s.get_state()
+        for dr, nbins in ((0.0025, 1500), (0.01, 300), (0.005, 300)):
+            g = s.rdf(dr, nbins, reset=(nbins > 300))
+            ref = [oracle.rdf(p[off[k]:off[k + 1]], types[k], Ls[k], dr, nbins) for k in range(3)]
+            assert np.allclose(g, np.mean(ref, axis=0), rtol=1e-12, atol=0)
+            assert np.allclose(s.rdf(dr, nbins), g, rtol=1e-12, atol=0)
