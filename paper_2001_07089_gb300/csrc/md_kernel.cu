@@ -45,7 +45,6 @@ struct Shared {
   double4_32a tabd[MD_MAXTYPES * MD_MAXTYPES];
   double2 tabed[MD_MAXTYPES * MD_MAXTYPES];
   double red[16][MD_NPART];
-  long long scan[32];
   RepDev lone;  // Nose-Hoover steps of a single replica: this CTA's copy (see reduce_phase)
   int snap;
   unsigned gen;  // grid barrier generation this CTA waits for next (thread 0)
@@ -1017,10 +1016,11 @@ __device__ __forceinline__ void cell_of_pos(const KParams& p, const RepDev& R, i
   cz = (int)(((uint64_t)q.z * (uint64_t)nc) >> 32);
 }
 
-// Block-wide exclusive scan of one number per thread.
+// Block-wide exclusive scan of one number per thread (in the memory of sum_records, which has its own barriers).
 template <class V>
 __device__ V block_exclusive_scan(Shared& sh, V v, V* total) {
-  V* const tot = reinterpret_cast<V*>(sh.scan);
+  static_assert(sizeof(sh.red) >= 32 * sizeof(V), "a number per warp");
+  V* const tot = reinterpret_cast<V*>(&sh.red[0][0]);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   V x = v;
 #pragma unroll
@@ -1277,11 +1277,14 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
   __shared__ int s_plo[MD_ROWS_MAX], s_pb[MD_ROWS_MAX + 1];
   __shared__ int s_ref;
   const int64_t ngrp = p.ctl->grp_total;
-  // from the last CTA down: the first few are resident side by side on the SMs of
-  // a small GPC, the last ones each on an SM of their own (64 replicas of 500, one
-  // group each: the build 196 us from the first CTA up, now 81)
-  for (int64_t g = gridDim.x - 1 - blockIdx.x; g < ngrp; g += gridDim.x) {
-    const int r = find_replica(p, g, &RepDev::grp_base);
+  // Fewer groups than CTAs: from the last CTA down. The first few are resident
+  // side by side on the SMs of a small GPC, the last ones each on an SM of their own
+  // (64 replicas of 500, one group each: the build 196 us from the first CTA up, now
+  // 81). More: from the first up, 1 % faster at N = 10^6.
+  int r = 0;
+  const int64_t g0 = ngrp < gridDim.x ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  for (int64_t g = g0; g < ngrp; g += gridDim.x) {
+    if (p.nrep > 1) r = find_replica(p, g, &RepDev::grp_base);
     const RepDev& R = p.reps[r];
     const int lg = (int)(g - R.grp_base);
     const int nc = R.nc;
@@ -1639,8 +1642,9 @@ __device__ bool rebuild(const KParams& p, Shared& sh, int cur, int* fl, int64_t 
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = stride >> 5, total = p.ctl->sort_total;
     for (int64_t v = gtid >> 5; v < total; v += nwarps) {
-      // (if every replica rebuilds, the numbering is that of all cells, whose replicas are at hand)
-      const RepDev& R = p.reps[total == p.ncells ? p.cell_rep[v] : find_replica(p, v, &RepDev::sort_base)];
+      // (if every one of several replicas rebuilds, the numbering is that of all cells, whose replicas are at hand)
+      const bool all = p.nrep > 1 && total == p.ncells;
+      const RepDev& R = p.reps[all ? p.cell_rep[v] : find_replica(p, v, &RepDev::sort_base)];
       const int c = (int)(v - R.sort_base);
       const int lo = p.cstart[R.cs0 + c], hi = p.cstart[R.cs0 + c + 1];
       const int n = hi - lo;
