@@ -885,8 +885,8 @@ __device__ void sum_records(Shared& sh, const double* part, int64_t stride, int6
 // update that needs them; CTA 0 also writes the replica. What bounds small
 // systems is the barriers (about 2 us each with the phase's latency): 50
 // steps of 1000 particles in a plane 1046 -> 931 us, of N = 10^6 17.86 ->
-// 17.70 ms. At 304 CTAs the repeated reads are 20 MB from L2 at most (the
-// largest system reduced in one level). With several replicas a CTA's
+// 17.70 ms. At 304 CTAs the repeated reads are 20 MB per quantity from L2 at most
+// (the largest system reduced in one level). With several replicas a CTA's
 // particles belong to many of them, and the barrier stays.
 template <bool MIX>
 __device__ bool reduce_phase(const KParams& p, Shared& sh, const double* part, int upt, int mode, int64_t step,
@@ -1389,10 +1389,9 @@ __device__ __forceinline__ void build_lists(const KParams& p, Shared& sh, int cu
     const uint4 ref = p.pq[cur][s_ref];
     {
       // two candidates per thread and turn, both loads in flight together. (The
-      // loads are made whether or not there is a second candidate: with them
-      // under a condition, in an array, the compiler left the type word of the
-      // second one unset in some instances of this code, and candidates of type
-      // 1 were held to the radius of type 0.)
+      // loads are made whether or not there is a second candidate. A form with
+      // them under a condition, in an array, was seen to hold candidates of type 1
+      // to the radius of type 0 in some instances; why was not found out.)
       const uint4* __restrict__ pqc = p.pq[cur];
       const float sc = R.fxs;
       const int B = (int)blockDim.x;
