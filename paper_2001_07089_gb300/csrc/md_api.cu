@@ -413,6 +413,7 @@ struct RdfArgs {
   const uint4* xbq;   // positions at the last list build: the cells that slots are sorted by
   int32_t* unit;      // first slots of the units, replica r's from unit[off]
   int32_t* nunits;    // per replica
+  int32_t* nowhere;   // per replica: whether a particle's position is NaN (FP64; its words are those of some place)
   const int32_t* blk; // first CTA of each replica, and the number of CTAs (one replica: not read)
   const uint4* pq;
   const uint64_t* pfx;
@@ -556,6 +557,10 @@ __global__ void __launch_bounds__(RDF_LIST) k_rdf_units(RdfArgs a) {
   bool first = false;
   int layers;
   if (in && k < R.n) {
+    if (!a.mixed) {
+      const double4_32a x = a.p4[i];
+      if (isnan(x.x) || isnan(x.y) || isnan(x.z)) a.nowhere[r] = 1;
+    }
     if (!rdf_layers((a.dr * a.nbins + a.skin) * a.iunit, R.nc, R.cellw, &layers)) {
       first = k % RDF_PART == 0;
     } else if (k == 0 || i % RDF_CUT == 0) {
@@ -611,7 +616,8 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(RdfArgs a) {
   // at most `span`, and the words' own error
   const double span = rel ? (double)(RDF_CELLS + layers + 1) * (double)R.cellw : rmax;
   const double err = 1e-6 * span + 8.0 * (R.L * a.iunit) / 4294967296.0;
-  const float edge = (float)(err / dr + 1e-6 * a.nbins), invdr = (float)(1.0 / dr);
+  // (with a particle that is nowhere every pair is binned from the exact positions)
+  const float edge = a.nowhere[r] ? 1.0f : (float)(err / dr + 1e-6 * a.nbins), invdr = (float)(1.0 / dr);
   const float rmax2f = (float)((rmax + 2.0 * err) * (rmax + 2.0 * err) * (1.0 + 1e-6));
   RdfWarp& W = sh_w[warp];
   int head = 0, count = 0;  // the queue; head also counts the pairs binned since the last flush
@@ -1801,7 +1807,9 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
   // (two arrays of a rebuild, which has no use for them now: 32 entries per replica at least)
   a.unit = s->d_scat;
   a.nunits = s->d_cellof;
-  a.blk = s->d_cellof + s->nrep;
+  a.nowhere = s->d_cellof + s->nrep;
+  int32_t* const blk = s->d_cellof + 2 * (int64_t)s->nrep;
+  a.blk = blk;
   a.pq = s->d_pq[s->ctl.cur];
   a.pfx = s->d_pfx;
   a.p4 = s->d_p4[s->ctl.cur];
@@ -1829,9 +1837,9 @@ md_status md_rdf(md_system* s, double dr, int64_t nbins, double* g, int reset) {
     const int64_t fair = (int64_t)std::ceil(8.0 * s->nsm * work[r] / total);
     s->rdf_blk.push_back(s->rdf_blk.back() + (int32_t)std::max<int64_t>(1, std::min(most, fair)));
   }
-  CK(cudaMemsetAsync(a.nunits, 0, 4 * (size_t)s->nrep, s->stream));
+  CK(cudaMemsetAsync(a.nunits, 0, 8 * (size_t)s->nrep, s->stream));
   if (s->nrep > 1)
-    CK(cudaMemcpyAsync(s->d_cellof + s->nrep, s->rdf_blk.data(), 4 * s->rdf_blk.size(), cudaMemcpyHostToDevice, s->stream));
+    CK(cudaMemcpyAsync(blk, s->rdf_blk.data(), 4 * s->rdf_blk.size(), cudaMemcpyHostToDevice, s->stream));
   k_rdf_units<<<blocks_for(s->ntot, RDF_LIST), RDF_LIST, 0, s->stream>>>(a);
   CK(cudaGetLastError());
   k_rdf<<<(unsigned)s->rdf_blk.back(), 32 * RDF_WARPS, 0, s->stream>>>(a);

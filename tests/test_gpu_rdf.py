@@ -167,3 +167,19 @@ def test_uneven_batch_many_bins_and_accumulation(prec):
             ref = [oracle.rdf(p[off[k]:off[k + 1]], types[k], Ls[k], dr, nbins) for k in range(3)]
             assert np.allclose(g, np.mean(ref, axis=0), rtol=1e-12, atol=0)
             assert np.allclose(s.rdf(dr, nbins), g, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n,L", [(1000, 9.4), (3000, 40.0)])
+def test_a_particle_without_a_position_is_in_no_pair(n, L):
+    """FP64: the 32-bit words of a position that is not a number are those of some place; no pair is counted there."""
+    pos = wl.uniform_positions(n, L, 31)
+    pos[:200] = np.random.default_rng(2).uniform(-1.0, 1.0, (200, 3)) % L  # close to where a NaN's words are
+    pos[n // 2, 1] = np.nan
+    types = wl.ka_types(n, 31).astype(np.int32)
+    rest = np.arange(n) != n // 2
+    dr, nbins = 0.02, 200
+    with system(n, L, types, "fp64") as s:
+        s.set_state(pos)
+        g = s.rdf(dr, nbins, reset=True)
+    ref = counts(oracle.rdf(pos[rest], types[rest], L, dr, nbins), types[rest], L, dr, nbins)
+    assert np.array_equal(counts(g, types, L, dr, nbins), ref)
