@@ -215,7 +215,7 @@ __global__ void k_order(Scratch s) {
 // terms. Members of the 27 cells are read from memory once per cell instead of
 // once per particle and pair, and wrapped once. A candidate of an unknown type
 // makes every particle of the item NaN. Measured at n = 20 011 (the whole call):
-// 3093 us with one thread per particle walking the cells in FP64, 200 us so.
+// 3093 us with one thread per particle walking the cells in FP64, 190 us so.
 __global__ void __launch_bounds__(kForceThreads) k_forces(Scratch s, const double* __restrict__ pos,
                                                           const uint8_t* __restrict__ types, int n, int ntypes, int nc,
                                                           double L, Table tab, double* f, double* pe_out,
